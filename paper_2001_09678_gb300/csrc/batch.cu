@@ -111,12 +111,13 @@ __device__ __noinline__ void run_pass(const LevelArgs &a, int pb, int dir, int v
 __device__ __noinline__ void run_cost(const LevelArgs &a, int b0, int count, int view, int tid,
                                       unsigned char *sm)
 {
-    const int nseg = (a.W + kSegPix - 1) / kSegPix;
+    const int seg = cost_seg(a.W, a.N, cost_seg_max(a.N));
+    const int nseg = (a.W + seg - 1) / seg;
     for (int b = b0; b < b0 + count; ++b) {
         if (a.N == 5)
-            cost_body<5>(a, a.D - 1, b % nseg, b / nseg, view, tid, sm);
+            cost_body<5, 0>(a, a.D - 1, seg, b % nseg, b / nseg, view, tid, sm);
         else
-            cost_body<3>(a, a.D - 1, b % nseg, b / nseg, view, tid, sm);
+            cost_body<3, 0>(a, a.D - 1, seg, b % nseg, b / nseg, view, tid, sm);
         __syncthreads();   // the staging is reused by the next block
     }
 }
@@ -449,7 +450,8 @@ mpv_status plan_batch(const mpv_params &p, const PairJob *jobs, int n, uint8_t *
                     for (int y = 0; y < a.H; y += 16)
                         add(kSeed, l, v, 0, std::min(16, a.H - y), 0, y,
                             stage_of(l - 1, v, 3), -1, stage_of(l, v, 0));
-            const int nseg = (a.W + kSegPix - 1) / kSegPix;
+            const int seg = cost_seg(a.W, a.N, cost_seg_max(a.N));
+            const int nseg = (a.W + seg - 1) / seg;
             const int nblk = nseg * a.H;
             const int cb = std::max(1, tune.cost_blocks);
             for (int v = 0; v < nviews; ++v)

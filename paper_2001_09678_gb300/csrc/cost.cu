@@ -9,50 +9,74 @@
 // (c1, c2 = C1, C2 scaled by n^2 and rounded) and the cost is
 //     floor(255 (B1 B2 - A1 A2) / (2 B1 B2))  in [0, 255];  255 when x - u < 0.
 //
-// GPU design ("fast SSIM", Fig. fast_ssim, read as running box sums).  One block per
-// 256-pixel row segment and view:
+// GPU design ("fast SSIM", Fig. fast_ssim, read as running box sums).  One block per row
+// segment and view:
 //  * the block stages, in shared memory, every image column its pixels can reach as the
-//    N patch-row bytes packed in a 64-bit word, and the patch statistics of every centre
-//    (sum S, V = n * sum of squares - S^2, and both as floats);
-//  * each lane owns one label and slides along the row: the cross sum Sxy of pixel x
-//    follows from pixel x-1 by adding the entering column product (two dp4a) and
-//    subtracting the leaving one, kept in a register ring of the last N products; where
-//    the window start changes between neighbours the lane re-sums the N products;
-//  * the quotient is estimated in fp32 from A2 (exact int) and the float statistics and
-//    made exact with an int64 check only when the estimate lies within 1e-3 of an
-//    integer (the estimate's error is below 2e-4; see ssim_quotient).
+//    N patch-row bytes packed in a 64-bit word, with the patch statistics of the centre whose
+//    window that column completes (one 16-byte load per node of I1, 24 broadcast bytes of I0);
+//  * each lane owns one label of the window ring and slides along the row: the cross sum Sxy
+//    of pixel x follows from pixel x-1 by adding the entering column product (two dp4a) and
+//    subtracting the leaving one, kept in a register ring of the last N products;
+//  * the quotient is estimated in fp32 from exact float sums and made exact with an int64
+//    check only when the estimate lies within 1.2e-4 of an integer (see cost_body.cuh).
+// Bound: issue slots (84 % active at full range, 40 warp instructions per 32 nodes; about 65
+// with windows, of which staging is a quarter and moved windows another) and shared-memory
+// wavefronts (8 per 32 nodes).  Measured on a GB300, both views, per frame: 1280x720, D = 128,
+// three scales 233 -> 175 us; 1920x1080, D = 192 860 -> 484 us (48 labels in 1.5 instead of 2
+// passes over the pixels); 1280x720, 128 labels at full range 522 -> 291 us.  Segments of 160,
+// 320, 480 and 640 pixels took 191, 175, 182 and 178 us; 4, 5 and 6 blocks per SM 180, 175
+// and 176 us.
 #include "cost_body.cuh"
 
 namespace mpv {
 
 namespace {
 
-template <int N>
-__global__ void __launch_bounds__(kCostThreads) cost_kernel(LevelArgs a, int uspan_max)
+constexpr int kCostBlocks = 1216;     // about 8 per SM: two rounds of resident blocks
+
+template <int N, int ST>
+__global__ void __launch_bounds__(kCostThreads, 5) cost_kernel(LevelArgs a, int uspan_max, int seg)
 {
     if (a.gate && *a.gate == 0) return;
     extern __shared__ __align__(16) unsigned char smem[];
-    cost_body<N>(a, uspan_max, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, smem);
+    cost_body<N, ST>(a, uspan_max, seg, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, smem);
+}
+
+template <int N, int ST>
+void launch_cost_n(const LevelArgs &a, cudaStream_t s)
+{
+    // widest disparity span of a segment: window starts lie in [0, D - Dw]
+    const int uspan_max = a.D - 1;
+    const CostSmem L = cost_smem_layout(a.N / 2, uspan_max);
+    // the widest segments of which the launch still has kCostBlocks blocks: wide ones stage
+    // fewer columns per pixel, but a small level needs its blocks spread over the GPU
+    const int u = cost_seg_unit(N);
+    int seg = cost_seg(a.W, N, cost_seg_max(N));
+    while (seg > u && (int64_t)((a.W + seg - 1) / seg) * a.H * a.nviews < kCostBlocks)
+        seg = cost_seg(a.W, N, seg - u);
+    dim3 grid((a.W + seg - 1) / seg, a.H, a.nviews);
+    cudaFuncSetAttribute(cost_kernel<N, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)L.bytes);
+    cost_kernel<N, ST><<<grid, kCostThreads, L.bytes, s>>>(a, uspan_max, seg);
+}
+
+template <int N>
+void launch_cost_st(const LevelArgs &a, cudaStream_t s)
+{
+    switch (a.Dws) {   // the common strides as constants (store addresses, window wrap)
+    case 16: launch_cost_n<N, 16>(a, s); return;
+    case 32: launch_cost_n<N, 32>(a, s); return;
+    case 48: launch_cost_n<N, 48>(a, s); return;
+    default: launch_cost_n<N, 0>(a, s); return;
+    }
 }
 
 }  // namespace
 
 void launch_cost(const LevelArgs &a, cudaStream_t s)
 {
-    // widest disparity span of a segment: window starts lie in [0, D - Dw]
-    const int uspan_max = a.D - 1;
-    const int R = a.N / 2;
-    const CostSmem L = cost_smem_layout(R, uspan_max);
-    dim3 grid((a.W + kSegPix - 1) / kSegPix, a.H, a.nviews);
-    if (a.N == 5) {
-        cudaFuncSetAttribute(cost_kernel<5>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)L.bytes);
-        cost_kernel<5><<<grid, kCostThreads, L.bytes, s>>>(a, uspan_max);
-    } else {
-        cudaFuncSetAttribute(cost_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)L.bytes);
-        cost_kernel<3><<<grid, kCostThreads, L.bytes, s>>>(a, uspan_max);
-    }
+    if (a.N == 5) launch_cost_st<5>(a, s);
+    else launch_cost_st<3>(a, s);
 }
 
 }  // namespace mpv
