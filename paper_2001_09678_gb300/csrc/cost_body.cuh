@@ -2,7 +2,7 @@
 // (block index, thread index) shared by the stand-alone kernel and the batch
 // scheduler's persistent kernel.
 #pragma once
-#include "mpv_internal.cuh"
+#include "volume_layout.cuh"
 
 namespace mpv {
 
@@ -154,6 +154,8 @@ struct CostBlock {
                           // its sign bit, whether that differs from the previous pixel's
     int umax, nb, na;
     int Dw, Dws;
+    int stride;           // bytes per pixel of the cost volume
+    int nq;               // wide volumes: cost words per lane
     int imin;             // entries before it belong to matches left of the right image
     int c1, c2;
     int *err;
@@ -167,14 +169,15 @@ struct CostBlock {
 // pixel's products anew.  Sxy carries kRound23Bits, so that its bits are a float and no
 // conversion is needed.  Nodes whose estimate is too close to an integer are noted and
 // decided after each chunk of N pixels.  WIN: the level has windows.  EDGE: some matches fall
-// left of the right image or some labels are padding (cost 255).  ST: the volume's stride,
-// 0: B.Dws.
-template <int N, int ST, bool WIN, bool EDGE>
+// left of the right image or some labels are padding (cost 255).  ST: Dws as a constant, 0:
+// B.Dws.  WIDE: the wide byte order and stride (levels without windows).
+template <int N, int ST, bool WIDE, bool WIN, bool EDGE>
 __device__ __forceinline__ void cost_stream(const CostBlock &B, int xs, int xe, int slot,
                                             uint8_t *out)
 {
     constexpr int R = N / 2, n = N * N, NR = N;
     const int M = ST ? ST : B.Dws;
+    const int MS = WIDE ? B.stride : M;           // bytes per pixel
     const float c1f = (float)B.c1, c2f = (float)B.c2;
     auto window = [&](int x) { return (B.col0[x + 1 + 2 * R].y >> 16) & 0x3FFF; };
     auto label = [&](int lo) {   // rel
@@ -185,6 +188,7 @@ __device__ __forceinline__ void cost_stream(const CostBlock &B, int xs, int xe, 
     auto entry_off = [&](int lo, int rel) {
         return 1 + 2 * R + B.umax - lo - (EDGE ? min(rel, B.Dw - 1) : rel);
     };
+    auto byte_of = [&](int rel) { return WIDE ? wide_byte(rel, B.nq) : rel; };
     // the integers of one node; exact cost
     auto exact_node = [&](int x) {
         const int lo = window(x), rel = label(lo), off = entry_off(lo, rel);
@@ -207,7 +211,7 @@ __device__ __forceinline__ void cost_stream(const CostBlock &B, int xs, int xe, 
             const float den = fmaf((float)sy, (float)sy, s0.z) * (s0.w + (float)vy);
             q = ssim_exact((int)(127.5f - 127.5f * (num / den)), A2, sx, vx, sy, vy, B.c1, B.c2);
         }
-        out[x * M + rel] = (uint8_t)q;
+        out[x * MS + byte_of(rel)] = (uint8_t)q;
     };
 
     const int xc = xs + (xe - xs) / NR * NR;      // whole chunks end here
@@ -238,7 +242,7 @@ __device__ __forceinline__ void cost_stream(const CostBlock &B, int xs, int xe, 
         const int2 *c0 = B.col0 + xs + 1 + 2 * R;   // entering I0 column of the chunk's first
         const int4 *e = B.e1 + xs + off;            // pixel, and its I1 entry
         const float4 *st = B.st0 + xs;
-        unsigned po = (unsigned)(xs * M + rel);
+        unsigned po = (unsigned)(xs * MS + byte_of(rel));
         int pad = EDGE ? (rel < B.Dw ? B.imin : 0x7FFFFFFF) - off : 0;
         for (int xb = xs; xb < xc; xb += NR) {
             unsigned bad = 0;
@@ -248,7 +252,7 @@ __device__ __forceinline__ void cost_stream(const CostBlock &B, int xs, int xe, 
                 if (WIN && a.y < 0) {   // the window moved
                     const int lo = (a.y >> 16) & 0x3FFF;
                     const int r = label(lo), o = entry_off(lo, r);
-                    po += (unsigned)(r - rel);
+                    po += (unsigned)(r - rel);      // (windows: not WIDE)
                     rel = r;
                     if (o != off) {
                         e += o - off;
@@ -280,12 +284,12 @@ __device__ __forceinline__ void cost_stream(const CostBlock &B, int xs, int xe, 
                 if (fabsf(t - (m - kRound23)) > kQuotientSafe) bad |= 1u << j;
                 int q = __float_as_int(m);
                 if (EDGE) q = xb + j < pad ? 255 : q;
-                out[po + (unsigned)(j * M)] = (uint8_t)q;
+                out[po + (unsigned)(j * MS)] = (uint8_t)q;
             }
             c0 += NR;
             e += NR;
             st += NR;
-            po += (unsigned)(NR * M);
+            po += (unsigned)(NR * MS);
             while (bad) {
                 exact_node(xb + __ffs(bad) - 1);
                 bad &= bad - 1;
@@ -297,7 +301,7 @@ __device__ __forceinline__ void cost_stream(const CostBlock &B, int xs, int xe, 
 
 // One block of the cost kernel: row segment bx (of seg pixels), row by, view bz; smem: the
 // block's dynamic shared memory (cost_smem_layout bytes).
-template <int N, int ST>
+template <int N, int ST, bool WIDE>
 __device__ __forceinline__ void cost_body(const LevelArgs &a, int uspan_max, int seg, int bx,
                                           int by, int bz, int tid, unsigned char *smem)
 {
@@ -318,7 +322,17 @@ __device__ __forceinline__ void cost_body(const LevelArgs &a, int uspan_max, int
     uint2 *col0 = (uint2 *)(smem + L.off_col0);
     const int lane = tid & 31, warp = tid >> 5;
 
-    if (a.zero_s) {   // this segment's summed energies start at zero (16-byte stores)
+    const int stride = WIDE ? 4 * a.wide_g * a.wide_nq : Dws;
+    if (WIDE) {   // this segment's byte sums start at zero, the bytes of no label at cost 255
+        const int64_t at = ((int64_t)y * W + x0) * stride;     // a multiple of 32
+        const int n16 = npx * (stride / 16);
+        uint4 *ez = (uint4 *)(V.E + at), *cz = (uint4 *)(V.C + at);
+        const uint32_t f = 0xFFFFFFFFu;
+        for (int i = tid; i < n16; i += kCostThreads) {
+            ez[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (Dws < stride) cz[i] = make_uint4(f, f, f, f);
+        }
+    } else if (a.zero_s) {   // this segment's summed energies start at zero (16-byte stores)
         uint4 *sz = (uint4 *)(V.S + ((int64_t)y * W + x0) * Dws);
         const int n16 = npx * Dws / 8;     // Dws is a multiple of 16
         for (int i = tid; i < n16; i += kCostThreads) sz[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -386,11 +400,11 @@ __device__ __forceinline__ void cost_body(const LevelArgs &a, int uspan_max, int
     __syncthreads();
 
     // (the entry of the centre at the image's first column lies R columns past it)
-    const CostBlock B{e1, st0, (const int2 *)col0, umax, nb, na, Dw, Dws, R - b0, a.c1, a.c2, a.err};
+    const CostBlock B{e1, st0, (const int2 *)col0, umax, nb, na, Dw, Dws, stride, a.wide_nq, R - b0, a.c1, a.c2, a.err};
     // 32 labels of one pixel per warp step; a last group of 16 labels as two streams, half of
     // the warp's pixels each (48 labels in 1.5 passes over the pixels instead of 2)
     const int per_warp = seg / kCostWarps;
-    uint8_t *out = V.C + ((int64_t)y * W + x0) * Dws;
+    uint8_t *out = V.C + ((int64_t)y * W + x0) * stride;
     const bool edge = x0 - umax < 0 || Dw < Dws;
     for (int k0 = 0; k0 < Dws; k0 += 32) {
         const int half = Dws - k0 < 32;      // a group of 16
@@ -398,12 +412,12 @@ __device__ __forceinline__ void cost_body(const LevelArgs &a, int uspan_max, int
         const int xs = warp * per_warp + (half && lane >= 16 ? len : 0);
         const int xe = min(xs + len, npx);
         const int slot = k0 + (half ? lane & 15 : lane);
-        if (V.lo) {
-            if (edge) cost_stream<N, ST, true, true>(B, xs, xe, slot, out);
-            else cost_stream<N, ST, true, false>(B, xs, xe, slot, out);
+        if (!WIDE && V.lo) {
+            if (edge) cost_stream<N, ST, false, true, true>(B, xs, xe, slot, out);
+            else cost_stream<N, ST, false, true, false>(B, xs, xe, slot, out);
         } else {
-            if (edge) cost_stream<N, ST, false, true>(B, xs, xe, slot, out);
-            else cost_stream<N, ST, false, false>(B, xs, xe, slot, out);
+            if (edge) cost_stream<N, ST, WIDE, false, true>(B, xs, xe, slot, out);
+            else cost_stream<N, ST, WIDE, false, false>(B, xs, xe, slot, out);
         }
     }
 }

@@ -53,6 +53,7 @@ struct ViewLevel {
     uint16_t *d;             // pre-check WTA map [H][W]
     const uint16_t *S2;      // layered merge: the final layer's second pass (WTA and the
                              // stage dump read floor((S + S2) / 2)); nullptr otherwise
+    uint8_t *E;              // byte sums [H][W][bytes per pixel], in place of S; see below
 };
 
 struct LevelArgs {
@@ -74,6 +75,11 @@ struct LevelArgs {
     unsigned long long *edge;  // optional [2]: WTA at a window edge inside the range, pixels
     int block_cut;   // > 0: independent block_cut x block_cut tiles (scan paths restart)
     int zero_s;      // the cost kernel also clears S (the summed merge accumulates into it)
+    // Byte sums.  An energy is its cost plus E = M' - min_v L, 0 <= E <= T, so the sum over the
+    // paths is npaths C + sum E, and while npaths T <= 255 the directions add the E as bytes:
+    // half the bytes of 16-bit sums, which the reductions of wide pixels are bound by.
+    int wide_g;      // wide levels (agg_wide.cu): lanes per path, cost words per lane; C and E
+    int wide_nq;     // then have 4 wide_g wide_nq bytes per pixel.  0: C and S as above
     const int *gate; // optional device word: 0 = every kernel of this level returns at once
     int *err;        // bounds-checked builds: the device error word (see MPV_IN)
 };
@@ -123,6 +129,9 @@ void launch_pyramid2(const PyrJob *jobs, int njobs, int W, int H, cudaStream_t s
 void launch_seed(const SeedArgs &a, cudaStream_t s);
 void launch_cost(const LevelArgs &a, cudaStream_t s);
 void launch_aggregate(const LevelArgs &a, cudaStream_t s);
+// Whether the summed passes of a level without windows run on wide volumes, and their shape.
+bool wide_shape(const LevelArgs &a, int &G, int &NQ);
+void launch_wide(const LevelArgs &a, cudaStream_t s);
 
 // General passes (any radius and width, per-step penalties, layered merge).
 struct MergeArgs {
@@ -258,6 +267,7 @@ struct StageSink {
     uint16_t *lo = nullptr, *cost = nullptr, *disp = nullptr;
     uint32_t *sum = nullptr;
     float *proposal = nullptr;   // learned proposal: the network's top-level prediction
+    bool plain = false;          // keep the plain volume layout (the caller reads C itself)
 };
 
 bool params_valid(const mpv_params &p);
@@ -286,8 +296,9 @@ struct PairPlan {
 void plan_pair(const mpv_params &p, const PairJob &job, uint8_t *base, int nviews,
                bool level_volumes, PairPlan &pp);
 // Arguments of level l (both views) and of its window seeding (l > 0).
+// sums: the level may use byte sums (summed merge without a gradient table).
 LevelArgs level_args(const mpv_params &p, const PairPlan &pp, uint8_t *base, int l,
-                     const Tuning &tune, const int *gate);
+                     const Tuning &tune, const int *gate, bool sums = false);
 SeedArgs seed_args(const PairPlan &pp, uint8_t *base, int l, const int *gate,
                    int *err = nullptr);
 

@@ -208,6 +208,7 @@ mpv_status enqueue_features(const mpv_params &p, const PairJob &job, uint8_t *ba
     StageSink dbg;
     dbg.view = view;
     dbg.level = 0;
+    dbg.plain = true;
     const mpv_status st = enqueue_pair(q, job, base, s, nullptr, &dbg);
     if (st != MPV_OK) return st;
     const int top = g.S - 1;
@@ -283,7 +284,7 @@ void plan_pair(const mpv_params &p, const PairJob &job, uint8_t *base, int nview
 }
 
 LevelArgs level_args(const mpv_params &p, const PairPlan &pp, uint8_t *base, int l,
-                     const Tuning &tune, const int *gate)
+                     const Tuning &tune, const int *gate, bool sums)
 {
     const Geometry &g = pp.g;
     const Layout &L = pp.L;
@@ -320,6 +321,15 @@ LevelArgs level_args(const mpv_params &p, const PairPlan &pp, uint8_t *base, int
         vl.S = (uint16_t *)(base + L.Sl[v][l]);
         vl.d = (uint16_t *)(base + L.d[v][l]);
         vl.S2 = nullptr;
+        vl.E = nullptr;
+    }
+    if (sums && l == 0 && wide_shape(a, a.wide_g, a.wide_nq)) {
+        // C and E share the region of C and S (adjacent, 3 Dws bytes per pixel, no fewer than
+        // two wide volumes); E starts on 8 bytes
+        const size_t vol = (size_t)a.W * a.H * (4 * a.wide_g * a.wide_nq);
+        for (int v = 0; v < pp.nviews; ++v) a.v[v].E = a.v[v].C + vol;
+    } else {
+        a.wide_g = a.wide_nq = 0;
     }
     return a;
 }
@@ -432,7 +442,9 @@ mpv_status enqueue_pair(const mpv_params &p, const PairJob &job, uint8_t *base, 
     if (!dbg && learned) cudaMemsetAsync(edge, 0, 2 * sizeof(unsigned long long), s);
     for (int l = 0; l <= last; ++l) {
         if (learned && l > 0 && l < top) continue;
-        LevelArgs a = level_args(p, pp, base, l, tune, gate);
+        // (the network's features read the top level's plain volume)
+        const bool sums = !layered && !grad_lut && !(learned && l == 0) && !(dbg && dbg->plain);
+        LevelArgs a = level_args(p, pp, base, l, tune, gate, sums);
         a.edge = (learned && l == top) ? edge : nullptr;
         if (learned && l == top) {
             // windows of the finest level from the network's prediction at the top level
@@ -526,6 +538,8 @@ mpv_status enqueue_pair(const mpv_params &p, const PairJob &job, uint8_t *base, 
                 m.double_up_dir = -1;
                 m.lut = grad_lut;
                 launch_aggregate_general(a, m, s);
+            } else if (a.wide_nq) {
+                launch_wide(a, s);
             } else {
                 launch_aggregate(a, s);
             }

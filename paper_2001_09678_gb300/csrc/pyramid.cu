@@ -5,6 +5,7 @@
 // centre comes from the coarser level's disparities, doubled (the sampling rate), as a
 // block mode at intermediate levels and by linear interpolation at the finest level.
 #include "pyramid_body.cuh"
+#include "volume_layout.cuh"
 
 namespace mpv {
 
@@ -51,6 +52,72 @@ __global__ void wta_kernel(LevelArgs a)
 {
     if (a.gate && *a.gate == 0) return;
     wta_body<LPP>(a, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, blockIdx.z);
+}
+
+// Winner-take-all on wide volumes (agg_wide.cu): S = npaths C + E, ties to the smallest
+// disparity.  Four threads per pixel, each with the G NQ consecutive bytes of G / 4 lanes.
+// Bound by DRAM (1280x720, 128 labels, both views: 472 MB in 90 us).
+template <int G, int NQ>
+__global__ void __launch_bounds__(256) wide_wta_kernel(LevelArgs a)
+{
+    if (a.gate && *a.gate == 0) return;
+    constexpr int R = 4 * G * NQ, TPP = 4, NW = G * NQ / 4;   // words per thread
+    const ViewLevel &v = a.v[blockIdx.z];
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = g / TPP;
+    const int sub = (int)(g % TPP);
+    uint32_t best = 0xFFFFFFFFu;
+    const bool in = i < (int64_t)a.W * a.H;
+    if (in) {
+        const uint8_t *pc = v.C + i * R + sub * (4 * NW), *pe = v.E + i * R + sub * (4 * NW);
+        uint32_t qc[NW], qe[NW];
+        if (NW % 4 == 0) {
+#pragma unroll
+            for (int k = 0; k < NW / 4; ++k) {
+                const uint4 x = ((const uint4 *)pc)[k], y = ((const uint4 *)pe)[k];
+                qc[4 * k] = x.x, qc[(4 * k + 1) % NW] = x.y;
+                qc[(4 * k + 2) % NW] = x.z, qc[(4 * k + 3) % NW] = x.w;
+                qe[4 * k] = y.x, qe[(4 * k + 1) % NW] = y.y;
+                qe[(4 * k + 2) % NW] = y.z, qe[(4 * k + 3) % NW] = y.w;
+            }
+        } else if (NW % 2 == 0) {
+#pragma unroll
+            for (int k = 0; k < NW / 2; ++k) {
+                const uint2 x = ((const uint2 *)pc)[k], y = ((const uint2 *)pe)[k];
+                qc[2 * k] = x.x, qc[(2 * k + 1) % NW] = x.y;
+                qe[2 * k] = y.x, qe[(2 * k + 1) % NW] = y.y;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < NW; ++k) {
+                qc[k] = ((const uint32_t *)pc)[k];
+                qe[k] = ((const uint32_t *)pe)[k];
+            }
+        }
+        const uint32_t np = (uint32_t)a.npaths << 16;
+#pragma unroll
+        for (int k = 0; k < NW; ++k)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const uint32_t c = (qc[k] >> (8 * b)) & 0xFFu, e = (qe[k] >> (8 * b)) & 0xFFu;
+                const int ln = (4 * k + b) / (4 * NQ), j = 4 * k + b - ln * 4 * NQ;
+                const int u = sub * (4 * NW) + ln * 4 * NQ + (j >> 1) + (j & 1) * 2 * NQ;
+                const uint32_t key = c * np + ((e << 16) | (uint32_t)u);
+                if (u < a.Dw) best = min(best, key);
+            }
+    }
+#pragma unroll
+    for (int o = 1; o < TPP; o <<= 1) best = min(best, __shfl_xor_sync(0xFFFFFFFFu, best, o));
+    if (in && sub == 0) v.d[i] = (uint16_t)(best & 0xFFFFu);
+}
+
+template <int NQ>
+void launch_wide_wta(const LevelArgs &a, cudaStream_t s)
+{
+    const int64_t nthreads = 4 * (int64_t)a.W * a.H;
+    const dim3 grid((unsigned)((nthreads + 255) / 256), 1, a.nviews);
+    if (a.wide_g == 4) wide_wta_kernel<4, NQ><<<grid, 256, 0, s>>>(a);
+    else wide_wta_kernel<8, NQ><<<grid, 256, 0, s>>>(a);
 }
 
 // Window-edge hits of the learned proposal: pixels whose minimum sits on an edge of
@@ -103,6 +170,12 @@ __global__ void unpack_kernel(LevelArgs a, int view, uint16_t *cost, uint32_t *s
     const int64_t pix = e / a.Dw;
     const int k = (int)(e - pix * a.Dw);
     const ViewLevel &v = a.v[view];
+    if (a.wide_nq) {
+        const int64_t j = pix * (4 * a.wide_g * a.wide_nq) + wide_byte(k, a.wide_nq);
+        if (cost) cost[e] = v.C[j];
+        if (sum) sum[e] = (uint32_t)a.npaths * v.C[j] + v.E[j];
+        return;
+    }
     if (cost) cost[e] = v.C[pix * a.Dws + k];
     if (sum) {
         const int64_t j = pix * a.Dws + k;
@@ -156,6 +229,15 @@ void launch_seed(const SeedArgs &a, cudaStream_t s)
 
 void launch_wta(const LevelArgs &a, cudaStream_t s)
 {
+    switch (a.wide_nq) {
+    case 0: break;
+    case 3: launch_wide_wta<3>(a, s); return;
+    case 4: launch_wide_wta<4>(a, s); return;
+    case 5: launch_wide_wta<5>(a, s); return;
+    case 6: launch_wide_wta<6>(a, s); return;
+    case 7: launch_wide_wta<7>(a, s); return;
+    default: launch_wide_wta<8>(a, s); return;
+    }
     const int lpp = a.Dws >= 32 ? 4 : 2;
     const int64_t nthreads = lpp * (int64_t)a.W * a.H;
     dim3 grid((unsigned)((nthreads + 255) / 256), 1, a.nviews);
