@@ -138,6 +138,10 @@ __device__ __forceinline__ void store_normalised(uint16_t *dst, const uint32_t (
 // continue the sweeps linearly from its edge, capped.
 // XM: the path minimum through shared memory instead of shuffles (8-lane paths; chosen at
 // dispatch where measured faster).
+// BS: byte sums (see LevelArgs) - the pass adds E = M' - min_v A into V.E, four labels per
+// word, instead of the energies into S.  With 12 labels per lane (KW = 6) the bytes of C and E
+// are ordered so that a lane's first 8 labels and its last 4 are one load and one reduction
+// each (bytes48_of).  PD: the level may have padding labels.
 // Shared memory of one block of agg_stencil_body: the re-indexing buffers (rbuf; sbuf for
 // the doubled pass of a layer), the gradient table (slut) and the path minima (redbuf).
 template <int G, int KW, int RM, bool WIN, bool LAYER, bool SWP, int NW>
@@ -147,8 +151,16 @@ struct StencilSmem {
     static constexpr int DWP = G * 2 * KW;
     static constexpr int PAD = (DWP + 4 * HW + 2 + 7) / 8 * 8;
     static constexpr int BUF = 2 * PAD + DWP;
-    static constexpr int nr = WIN ? NW * kPathsPerWarp * BUF : 8;              // uint16
-    static constexpr int ns = WIN && LAYER && !SWP ? NW * kPathsPerWarp * BUF : 8;
+    // a path's buffer starts on a multiple of 32 words plus skew(path), so that the words of
+    // the warp's lanes (KW apart) fall into different banks while their windows move alike
+    static constexpr int PATHW = (BUF / 2 + 31) / 32 * 32;
+    static constexpr int WARPW = kPathsPerWarp * PATHW + 32;
+    static constexpr int nr = WIN ? NW * WARPW * 2 : 8;                        // uint16
+    static constexpr int ns = WIN && LAYER && !SWP ? NW * WARPW * 2 : 8;
+    __host__ __device__ static constexpr int path_at(int warp, int path)       // in uint16
+    {
+        return 2 * (warp * WARPW + path * PATHW + path % KW + path / KW * (G * KW) % 32);
+    }
     static constexpr int nl = SWP ? 256 : 1;                                   // int
     static constexpr int nm = 2 * NW * 32;                                     // uint32
     // byte offsets in one 16-byte aligned block
@@ -158,7 +170,8 @@ struct StencilSmem {
     static constexpr size_t bytes = off_m + 4 * (size_t)nm;
 };
 
-template <int G, int KW, int RM, bool WIN, bool BLK, bool LAYER, bool SWP, bool XM, int NW>
+template <int G, int KW, int RM, bool WIN, bool BLK, bool LAYER, bool SWP, bool XM, int NW,
+          bool BS = false, bool PD = true>
 __device__ __forceinline__ void agg_stencil_body(const LevelArgs &a, const MergeArgs &mg, int bx,
                                                  int by, int bz, int tid, unsigned char *smem)
 {
@@ -202,8 +215,8 @@ __device__ __forceinline__ void agg_stencil_body(const LevelArgs &a, const Merge
     const int path = (bx * NW + warp) * kPathsPerWarp + grp;
     const ViewLevel &V = a.v[view];
 
-    uint16_t *gb = rbuf + (WIN ? (warp * kPathsPerWarp + grp) * BUF : 0);
-    uint16_t *sb = sbuf + (WIN && LAYER && !SWP ? (warp * kPathsPerWarp + grp) * BUF : 0);
+    uint16_t *gb = rbuf + (WIN ? SM::path_at(warp, grp) : 0);
+    uint16_t *sb = sbuf + (WIN && LAYER && !SWP ? SM::path_at(warp, grp) : 0);
     if (WIN) {
         for (int i = gl; i < BUF; i += kG) gb[i] = (uint16_t)kInf16;
         if (LAYER && !SWP)
@@ -223,7 +236,7 @@ __device__ __forceinline__ void agg_stencil_body(const LevelArgs &a, const Merge
     const uint32_t Tcap = Tx2 * up;
 
     // labels at or beyond Dw are padding: never a predecessor, never summed
-    const bool padded = Dw < DWP;
+    const bool padded = PD && Dw < DWP;
     uint32_t keep[KW];
 #pragma unroll
     for (int i = 0; i < KW; ++i) {
@@ -239,8 +252,9 @@ __device__ __forceinline__ void agg_stencil_body(const LevelArgs &a, const Merge
     const int nmax = __reduce_max_sync(kFull, n);
     const int pix0 = y0 * W + x0;
     const int dpix = dy * W + dx;
-    const uint8_t *cbase = V.C + gl * K;
+    const uint8_t *cbase = V.C + (BS && KW == 6 ? gl * 8 : gl * K);
     uint16_t *sbase = V.S + gl * K;
+    uint8_t *ebase = BS ? V.E + (KW == 6 ? gl * 8 : gl * K) : nullptr;
     const uint16_t *lob = V.lo;
 
     // prefetch ring (registers): cost bytes (or the previous layer's two words per
@@ -284,6 +298,11 @@ __device__ __forceinline__ void agg_stencil_body(const LevelArgs &a, const Merge
                 }
             } else if (KW == 1) {
                 cq[slot][0] = ld_pin_u16(src);
+            } else if (BS && KW == 6) {
+                const uint2 v = ld_pin_u64(src);
+                cq[slot][0] = v.x;
+                cq[slot][1 % CW] = v.y;
+                cq[slot][2 % CW] = ld_pin_u32(src + 32 - 4 * gl);
             } else if (CW % 2 == 0) {
 #pragma unroll
                 for (int j = 0; j < CW; j += 2) {
@@ -472,7 +491,12 @@ __device__ __forceinline__ void agg_stencil_body(const LevelArgs &a, const Merge
                 // words below e hold smaller labels: jumps up into (u, u+1); the cap
                 // (which waits for the path minimum) enters last
                 uint32_t m;
-                if constexpr (!LAYER) {
+                if constexpr (BS && G * KW == 16) {
+                    // the neighbours with their penalties added on the other pipe, then
+                    // 3-input minima: half the ALU instructions (slower with more words)
+                    m = __vimin3_u16x2(E[e], SH[e - 1] + E1, SH[e] + E1);
+                    m = __vimin3_u16x2(m, E[e - 1] + E2, E[e + 1] + E2);
+                } else if constexpr (!LAYER) {
                     // equal slopes both ways: the two neighbours d labels away share
                     // their penalty, min(A(u-d), A(u+d)) + eps(d) (no half reaches 2^16)
                     m = __viaddmin_u16x2(__vminu2(SH[e - 1], SH[e]), E1, E[e]);
@@ -495,6 +519,13 @@ __device__ __forceinline__ void agg_stencil_body(const LevelArgs &a, const Merge
                 }
                 if (asym) m = __viaddmin_u16x2(SA[i], Tx2, m);
                 m = __vminu2(m, cap);
+                if constexpr (BS) {
+                    const uint32_t e = m - m2;   // per half: no borrow, at most T
+                    A[i] = c[i] + e;
+                    if (padded) A[i] |= INF2 & ~keep[i];
+                    c[i] = e;
+                    continue;
+                }
                 uint32_t L = c[i] + m - m2;      // per half: no carry, no borrow
                 if (padded) {
                     L &= keep[i];
@@ -614,7 +645,19 @@ __device__ __forceinline__ void agg_stencil_body(const LevelArgs &a, const Merge
             }
         }
         if (act && !OUTN && MPV_IN(a.err, pix >= 0 && pix < W * H, 7)) {
-            if (KW % 2 == 0) {
+            if constexpr (BS) {
+                // the increments as bytes, four labels per word (padding labels' are ignored)
+                static_assert(KW == 2 || KW == 4 || KW == 6, "");
+                uint32_t w[KW / 2];
+#pragma unroll
+                for (int j = 0; j < KW / 2; ++j) w[j] = __byte_perm(c[2 * j], c[2 * j + 1], 0x6420);
+                uint8_t *ep = ebase + (int64_t)pix * DWP;
+                if (KW >= 4)
+                    atomicAdd((unsigned long long *)ep,
+                              ((unsigned long long)w[1 % (KW / 2)] << 32) | w[0]);
+                if (KW == 2) atomicAdd((unsigned int *)ep, w[0]);
+                if (KW == 6) atomicAdd((unsigned int *)(ep + 32 - 4 * gl), w[2 % (KW / 2)]);
+            } else if (KW % 2 == 0) {
                 unsigned long long *sp = (unsigned long long *)(sbase + (int64_t)pix * DWP);
 #pragma unroll
                 for (int j = 0; j < KW / 2; ++j)
@@ -685,7 +728,7 @@ __device__ __forceinline__ void agg_row_body(const LevelArgs &a, int bx, int vie
     const uint8_t *cp = V.C + pix0 * DWP + gl * K;
     uint16_t *sp = V.S + pix0 * DWP + gl * K;
     const uint16_t *lp = WIN ? V.lo + pix0 : nullptr;
-    uint16_t *gb = (uint16_t *)smem + (WIN ? (warp * PPW + grp) * BUF : 0);
+    uint16_t *gb = (uint16_t *)smem + (WIN ? SM::path_at(warp, grp) : 0);
     uint32_t *redbuf = (uint32_t *)(smem + SM::off_m);
     if (WIN) {
         for (int i = gl; i < BUF; i += kG) gb[i] = (uint16_t)kInf16;

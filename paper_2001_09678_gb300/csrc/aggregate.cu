@@ -12,7 +12,7 @@
 // and keeps every value small (at most 255 + T per pass); each pass adds L into the summed
 // volume S, or, in the paper's layered merge, stores it min-normalised for the next layer.
 //
-// Three kernels:
+// Kernels:
 //  * agg_stencil: 4 or 8 lanes own one scan path, each lane 2*KW consecutive labels packed
 //    two per 32-bit register (16-bit energies, absent labels = the sentinel 16384).  When
 //    the truncation makes every jump of more than R labels cost T (R = ceil(T/p1) - 1 <= 4;
@@ -28,37 +28,44 @@
 //    runs one layer of the layered merge (Section 3.2), the left-to-right pass with doubled
 //    upward jumps included; its sweep mode runs gradient-weighted slopes (Eq. EU) as
 //    untruncated packed sweeps.
+//  * byte sums (launch_bytes): the same passes where the sums of the energies' increments fit
+//    bytes (8 paths: T <= 31) and jumps beyond 2 labels are truncated, the usual case; the
+//    row directions in agg_rows.cuh, wide levels without windows in agg_wide.cu.
 //  * agg_scan8: 8 lanes per path, int32 labels, the two sweeps as segmented prefix and
 //    suffix minima across the lanes: the gradient and layered variants outside the packed
 //    kernel's bounds or widths.
 //  * agg_general: any window width: one warp per scan path, the sweeps written as prefix
 //    minima  min_{v<=u} A(v) + p1 (u-v) = p1 u + min_{v<=u} (A(v) - p1 v)  (and the mirror
 //    image), evaluated by shuffle scans over the lanes.
-#include "agg_stencil.cuh"
+#define MIN3 1
+#ifndef MIXDYN
+#define MIXDYN 0
+#endif
+#include "agg_rows.cuh"
 
 namespace mpv {
 
 namespace {
 
-template <int G, int KW, int RM, bool WIN, bool BLK, bool LAYER, bool SWP, bool XM>
+template <int G, int KW, int RM, bool WIN, bool BLK, bool LAYER, bool SWP, bool XM, bool BS>
 __global__ void __launch_bounds__(kStencilWarps * 32) agg_stencil(LevelArgs a, MergeArgs mg)
 {
     if (a.gate && *a.gate == 0) return;
     using SM = StencilSmem<G, KW, RM, WIN, LAYER, SWP, kStencilWarps>;
     __shared__ __align__(16) unsigned char smem[SM::bytes];
-    agg_stencil_body<G, KW, RM, WIN, BLK, LAYER, SWP, XM, kStencilWarps>(a, mg, blockIdx.x, blockIdx.y,
-                                                                       blockIdx.z, threadIdx.x, smem);
+    agg_stencil_body<G, KW, RM, WIN, BLK, LAYER, SWP, XM, kStencilWarps, BS>(
+        a, mg, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, smem);
 }
 
 template <int G, int KW, int RM, bool WIN, bool BLK, bool LAYER = false, bool SWP = false,
-          bool XM = false>
+          bool XM = false, bool BS = false>
 void launch_stencil(const LevelArgs &a, cudaStream_t s, const MergeArgs &mg = MergeArgs{},
                     int ndirs = 0)
 {
     const int maxp = a.W + a.H - 1;
     const int per_block = kStencilWarps * (32 / G);
     dim3 grid((maxp + per_block - 1) / per_block, ndirs ? ndirs : a.npaths, a.nviews);
-    agg_stencil<G, KW, RM, WIN, BLK, LAYER, SWP, XM><<<grid, kStencilWarps * 32, 0, s>>>(a, mg);
+    agg_stencil<G, KW, RM, WIN, BLK, LAYER, SWP, XM, BS><<<grid, kStencilWarps * 32, 0, s>>>(a, mg);
 }
 
 // The summed pass of the 8-lane shape with the row (horizontal) paths first: one 1-D grid
@@ -154,6 +161,7 @@ void launch_stencil_kw(const LevelArgs &a, cudaStream_t s)
 {
     const bool win = a.v[0].lo != nullptr;
     const bool blk = a.block_cut > 0;
+    // (16-bit sums: see launch_bytes for the rest)
     // the shared-memory path minimum: measured faster on 8 lanes of two words without
     // padding labels, slower with one word per lane or with padding
     if constexpr (G == 8 && KW == 2) {
@@ -800,8 +808,110 @@ int launch_layer(const LevelArgs &a, const MergeArgs &m, cudaStream_t s)
     return 1;
 }
 
+namespace {
+
+// Byte sums, label strides of 16 and 32: one grid, the row directions first (8 lanes per path,
+// agg_rows.cuh), then columns and diagonals with 4 lanes of 2 KW labels (agg_stencil_body), whose
+// labels are one load and one reduction per lane and step, a whole 32-byte sector per path of
+// 32 labels.  The rows set the time of small and middle levels (their steps wait on nothing
+// but their own arithmetic; 1237x371, 32 labels, windows: 111 ns per step alone, 149 ns with
+// register prefetch), issue slots that of large ones.  4 lanes halve the fixed work per path
+// of a step against 8; with 16-bit sums they lost, each reduction covering half a sector.
+// Measured on a GB300 per launch, 8 paths, both views, against 8 lanes with 16-bit sums:
+// 1280x720, 32 labels, windows 344 -> 267 us; 1237x371, 25 labels padded to 32 288 -> 172 us;
+// 640x480, 16 labels 146 -> 97 us.  Rows with the predecessor through shuffles and register
+// prefetch 275 us at 1280x720 (with 402 instead of 398 us per frame), 191 us at 1237x371; 4
+// lanes for the rows too 308 us; fewer resident blocks (2 to 4 per SM) slower.
+template <int G, int KW, bool WIN, bool PD>
+__global__ void __launch_bounds__(kStencilWarps * 32) agg_mixed(LevelArgs a, MergeArgs mg, int nhb,
+                                                              int ncb, int ndb)
+{
+    if (a.gate && *a.gate == 0) return;
+    constexpr int RKW = G * KW / 8;          // words per lane of the row passes' 8 lanes
+    using SR = RowSmem<RKW, WIN>;
+    using SC = StencilSmem<G, KW, 2, WIN, false, false, kStencilWarps>;
+    constexpr size_t rb = (size_t)SR::bytes * kStencilWarps;
+    __shared__ __align__(16) unsigned char smem[rb > SC::bytes ? rb : SC::bytes];
+    int b = blockIdx.x;
+    const int nrow = a.nviews * 2 * nhb;
+    if (b < nrow) {
+        const int view = b % a.nviews, r = b / a.nviews;
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        const int grp = (r >> 1) * kStencilWarps + warp;
+        if (r & 1) row_bytes_body<RKW, WIN, -1>(a, grp, view, lane, smem + warp * SR::bytes);
+        else row_bytes_body<RKW, WIN, 1>(a, grp, view, lane, smem + warp * SR::bytes);
+        return;
+    }
+    b -= nrow;
+    const int view = b % a.nviews;
+    b /= a.nviews;
+    int dir, bx;
+    if (b < 2 * ncb) {
+        dir = 2 + (b & 1);
+        bx = b >> 1;
+    } else {
+        b -= 2 * ncb;
+        dir = 4 + (b & 3);
+        bx = b >> 2;
+    }
+    agg_stencil_body<G, KW, 2, WIN, false, false, false, false, kStencilWarps, true, PD>(
+        a, mg, bx, dir, view, threadIdx.x, smem);
+}
+
+template <int G, int KW>
+void launch_mixed(const LevelArgs &a, cudaStream_t s)
+{
+    MergeArgs m{};
+    m.double_up_dir = -1;
+    constexpr int per = kStencilWarps * (32 / G);
+    const int nhb = (a.H + 4 * kStencilWarps - 1) / (4 * kStencilWarps), ncb = (a.W + per - 1) / per;
+    const int ndb = (a.W + a.H - 1 + per - 1) / per;
+    const int blocks = a.nviews * (2 * nhb + 2 * ncb + (a.npaths > 4 ? 4 * ndb : 0));
+    constexpr int th = kStencilWarps * 32;
+    if (a.Dw == a.Dws) {
+        if (a.v[0].lo) agg_mixed<G, KW, true, false><<<blocks, th, 0, s>>>(a, m, nhb, ncb, ndb);
+        else agg_mixed<G, KW, false, false><<<blocks, th, 0, s>>>(a, m, nhb, ncb, ndb);
+    } else {
+        if (a.v[0].lo) agg_mixed<G, KW, true, true><<<blocks, th, 0, s>>>(a, m, nhb, ncb, ndb);
+        else agg_mixed<G, KW, false, true><<<blocks, th, 0, s>>>(a, m, nhb, ncb, ndb);
+    }
+}
+
+template <int G, int KW>
+void launch_bytes_kw(const LevelArgs &a, cudaStream_t s)
+{
+    if (a.v[0].lo) launch_stencil<G, KW, 2, true, false, false, false, false, true>(a, s);
+    else launch_stencil<G, KW, 2, false, false, false, false, false, true>(a, s);
+}
+
+void launch_bytes(const LevelArgs &a, cudaStream_t s)
+{
+    switch (a.Dws) {
+    case 16: launch_mixed<4, 2>(a, s); return;
+    case 32: launch_mixed<4, 4>(a, s); return;
+    // (48 labels, 1920x1080 with windows: 2,088 -> 1,050 us, of which half the sums' bytes and
+    // whole-sector accesses (bytes48_of) are most; 123 instructions per step of 8 paths, L1
+    // 84 % busy)
+    case 48: launch_bytes_kw<4, 6>(a, s); return;
+    default: launch_bytes_kw<8, 4>(a, s); return;
+    }
+}
+
+}  // namespace
+
+// Jumps beyond two labels truncated, sums that fit a byte, no tiles.
+bool bytes_ok(const LevelArgs &a)
+{
+    return a.radius <= 2 && a.Dws <= 64 && a.block_cut == 0 &&
+           (int64_t)a.npaths * a.trunc <= 255 && packed_caps_ok(a, 1);
+}
+
 void launch_aggregate(const LevelArgs &a, cudaStream_t s)
 {
+    if (a.bytes) {
+        launch_bytes(a, s);
+        return;
+    }
     if (a.radius <= 4 && a.Dws <= 64 && packed_caps_ok(a, 1)) {
         const bool wide = a.lanes == kLanesWide;
         switch (a.Dws) {

@@ -115,9 +115,9 @@ __device__ __noinline__ void run_cost(const LevelArgs &a, int b0, int count, int
     const int nseg = (a.W + seg - 1) / seg;
     for (int b = b0; b < b0 + count; ++b) {
         if (a.N == 5)
-            cost_body<5, 0, false>(a, a.D - 1, seg, b % nseg, b / nseg, view, tid, sm);
+            cost_body<5, 0, 0>(a, a.D - 1, seg, b % nseg, b / nseg, view, tid, sm);
         else
-            cost_body<3, 0, false>(a, a.D - 1, seg, b % nseg, b / nseg, view, tid, sm);
+            cost_body<3, 0, 0>(a, a.D - 1, seg, b % nseg, b / nseg, view, tid, sm);
         __syncthreads();   // the staging is reused by the next block
     }
 }

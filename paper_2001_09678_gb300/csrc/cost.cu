@@ -34,15 +34,15 @@ namespace {
 
 constexpr int kCostBlocks = 1216;     // about 8 per SM: two rounds of resident blocks
 
-template <int N, int ST, bool WIDE>
+template <int N, int ST, int ORD>
 __global__ void __launch_bounds__(kCostThreads, 5) cost_kernel(LevelArgs a, int uspan_max, int seg)
 {
     if (a.gate && *a.gate == 0) return;
     extern __shared__ __align__(16) unsigned char smem[];
-    cost_body<N, ST, WIDE>(a, uspan_max, seg, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, smem);
+    cost_body<N, ST, ORD>(a, uspan_max, seg, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, smem);
 }
 
-template <int N, int ST, bool WIDE = false>
+template <int N, int ST, int ORD = 0>
 void launch_cost_n(const LevelArgs &a, cudaStream_t s)
 {
     // widest disparity span of a segment: window starts lie in [0, D - Dw]
@@ -55,22 +55,25 @@ void launch_cost_n(const LevelArgs &a, cudaStream_t s)
     while (seg > u && (int64_t)((a.W + seg - 1) / seg) * a.H * a.nviews < kCostBlocks)
         seg = cost_seg(a.W, N, seg - u);
     dim3 grid((a.W + seg - 1) / seg, a.H, a.nviews);
-    cudaFuncSetAttribute(cost_kernel<N, ST, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(cost_kernel<N, ST, ORD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)L.bytes);
-    cost_kernel<N, ST, WIDE><<<grid, kCostThreads, L.bytes, s>>>(a, uspan_max, seg);
+    cost_kernel<N, ST, ORD><<<grid, kCostThreads, L.bytes, s>>>(a, uspan_max, seg);
 }
 
 template <int N>
 void launch_cost_st(const LevelArgs &a, cudaStream_t s)
 {
     if (a.wide_nq) {
-        launch_cost_n<N, 0, true>(a, s);
+        launch_cost_n<N, 0, 1>(a, s);
         return;
     }
     switch (a.Dws) {   // the common strides as constants (store addresses, window wrap)
     case 16: launch_cost_n<N, 16>(a, s); return;
     case 32: launch_cost_n<N, 32>(a, s); return;
-    case 48: launch_cost_n<N, 48>(a, s); return;
+    case 48:
+        if (a.bytes) launch_cost_n<N, 48, 2>(a, s);
+        else launch_cost_n<N, 48>(a, s);
+        return;
     default: launch_cost_n<N, 0>(a, s); return;
     }
 }

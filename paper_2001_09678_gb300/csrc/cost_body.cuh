@@ -170,14 +170,15 @@ struct CostBlock {
 // conversion is needed.  Nodes whose estimate is too close to an integer are noted and
 // decided after each chunk of N pixels.  WIN: the level has windows.  EDGE: some matches fall
 // left of the right image or some labels are padding (cost 255).  ST: Dws as a constant, 0:
-// B.Dws.  WIDE: the wide byte order and stride (levels without windows).
-template <int N, int ST, bool WIDE, bool WIN, bool EDGE>
+// B.Dws.  ORD: byte order of a pixel - 0 by label, 1 the wide order and stride (levels without
+// windows), 2 the order of 48 labels with byte sums.
+template <int N, int ST, int ORD, bool WIN, bool EDGE>
 __device__ __forceinline__ void cost_stream(const CostBlock &B, int xs, int xe, int slot,
                                             uint8_t *out)
 {
     constexpr int R = N / 2, n = N * N, NR = N;
     const int M = ST ? ST : B.Dws;
-    const int MS = WIDE ? B.stride : M;           // bytes per pixel
+    const int MS = ORD == 1 ? B.stride : M;       // bytes per pixel
     const float c1f = (float)B.c1, c2f = (float)B.c2;
     auto window = [&](int x) { return (B.col0[x + 1 + 2 * R].y >> 16) & 0x3FFF; };
     auto label = [&](int lo) {   // rel
@@ -188,7 +189,9 @@ __device__ __forceinline__ void cost_stream(const CostBlock &B, int xs, int xe, 
     auto entry_off = [&](int lo, int rel) {
         return 1 + 2 * R + B.umax - lo - (EDGE ? min(rel, B.Dw - 1) : rel);
     };
-    auto byte_of = [&](int rel) { return WIDE ? wide_byte(rel, B.nq) : rel; };
+    auto byte_of = [&](int rel) {
+        return ORD == 1 ? wide_byte(rel, B.nq) : (ORD == 2 ? bytes48_of(rel) : rel);
+    };
     // the integers of one node; exact cost
     auto exact_node = [&](int x) {
         const int lo = window(x), rel = label(lo), off = entry_off(lo, rel);
@@ -252,7 +255,7 @@ __device__ __forceinline__ void cost_stream(const CostBlock &B, int xs, int xe, 
                 if (WIN && a.y < 0) {   // the window moved
                     const int lo = (a.y >> 16) & 0x3FFF;
                     const int r = label(lo), o = entry_off(lo, r);
-                    po += (unsigned)(r - rel);      // (windows: not WIDE)
+                    po += (unsigned)(byte_of(r) - byte_of(rel));
                     rel = r;
                     if (o != off) {
                         e += o - off;
@@ -301,7 +304,7 @@ __device__ __forceinline__ void cost_stream(const CostBlock &B, int xs, int xe, 
 
 // One block of the cost kernel: row segment bx (of seg pixels), row by, view bz; smem: the
 // block's dynamic shared memory (cost_smem_layout bytes).
-template <int N, int ST, bool WIDE>
+template <int N, int ST, int ORD>
 __device__ __forceinline__ void cost_body(const LevelArgs &a, int uspan_max, int seg, int bx,
                                           int by, int bz, int tid, unsigned char *smem)
 {
@@ -322,8 +325,8 @@ __device__ __forceinline__ void cost_body(const LevelArgs &a, int uspan_max, int
     uint2 *col0 = (uint2 *)(smem + L.off_col0);
     const int lane = tid & 31, warp = tid >> 5;
 
-    const int stride = WIDE ? 4 * a.wide_g * a.wide_nq : Dws;
-    if (WIDE) {   // this segment's byte sums start at zero, the bytes of no label at cost 255
+    const int stride = ORD == 1 ? 4 * a.wide_g * a.wide_nq : Dws;
+    if (ORD == 1) {   // this segment's byte sums start at zero, the bytes of no label at cost 255
         const int64_t at = ((int64_t)y * W + x0) * stride;     // a multiple of 32
         const int n16 = npx * (stride / 16);
         uint4 *ez = (uint4 *)(V.E + at), *cz = (uint4 *)(V.C + at);
@@ -332,6 +335,10 @@ __device__ __forceinline__ void cost_body(const LevelArgs &a, int uspan_max, int
             ez[i] = make_uint4(0u, 0u, 0u, 0u);
             if (Dws < stride) cz[i] = make_uint4(f, f, f, f);
         }
+    } else if (a.bytes) {
+        uint4 *ez = (uint4 *)(V.E + ((int64_t)y * W + x0) * Dws);
+        const int n16 = npx * Dws / 16;
+        for (int i = tid; i < n16; i += kCostThreads) ez[i] = make_uint4(0u, 0u, 0u, 0u);
     } else if (a.zero_s) {   // this segment's summed energies start at zero (16-byte stores)
         uint4 *sz = (uint4 *)(V.S + ((int64_t)y * W + x0) * Dws);
         const int n16 = npx * Dws / 8;     // Dws is a multiple of 16
@@ -412,12 +419,12 @@ __device__ __forceinline__ void cost_body(const LevelArgs &a, int uspan_max, int
         const int xs = warp * per_warp + (half && lane >= 16 ? len : 0);
         const int xe = min(xs + len, npx);
         const int slot = k0 + (half ? lane & 15 : lane);
-        if (!WIDE && V.lo) {
-            if (edge) cost_stream<N, ST, false, true, true>(B, xs, xe, slot, out);
-            else cost_stream<N, ST, false, true, false>(B, xs, xe, slot, out);
+        if (ORD != 1 && V.lo) {
+            if (edge) cost_stream<N, ST, ORD, true, true>(B, xs, xe, slot, out);
+            else cost_stream<N, ST, ORD, true, false>(B, xs, xe, slot, out);
         } else {
-            if (edge) cost_stream<N, ST, WIDE, false, true>(B, xs, xe, slot, out);
-            else cost_stream<N, ST, WIDE, false, false>(B, xs, xe, slot, out);
+            if (edge) cost_stream<N, ST, ORD, false, true>(B, xs, xe, slot, out);
+            else cost_stream<N, ST, ORD, false, false>(B, xs, xe, slot, out);
         }
     }
 }

@@ -78,6 +78,8 @@ struct LevelArgs {
     // Byte sums.  An energy is its cost plus E = M' - min_v L, 0 <= E <= T, so the sum over the
     // paths is npaths C + sum E, and while npaths T <= 255 the directions add the E as bytes:
     // half the bytes of 16-bit sums, which the reductions of wide pixels are bound by.
+    int bytes;       // 1: byte sums of the packed stencil, as many bytes per pixel as C (in the
+                     // order of bytes48_of for 48 labels)
     int wide_g;      // wide levels (agg_wide.cu): lanes per path, cost words per lane; C and E
     int wide_nq;     // then have 4 wide_g wide_nq bytes per pixel.  0: C and S as above
     const int *gate; // optional device word: 0 = every kernel of this level returns at once
@@ -130,6 +132,7 @@ void launch_seed(const SeedArgs &a, cudaStream_t s);
 void launch_cost(const LevelArgs &a, cudaStream_t s);
 void launch_aggregate(const LevelArgs &a, cudaStream_t s);
 // Whether the summed passes of a level without windows run on wide volumes, and their shape.
+bool bytes_ok(const LevelArgs &a);   // byte sums of the packed stencil apply
 bool wide_shape(const LevelArgs &a, int &G, int &NQ);
 void launch_wide(const LevelArgs &a, cudaStream_t s);
 

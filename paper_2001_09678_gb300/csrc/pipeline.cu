@@ -330,6 +330,9 @@ LevelArgs level_args(const mpv_params &p, const PairPlan &pp, uint8_t *base, int
         for (int v = 0; v < pp.nviews; ++v) a.v[v].E = a.v[v].C + vol;
     } else {
         a.wide_g = a.wide_nq = 0;
+        a.bytes = sums && bytes_ok(a);
+        if (a.bytes)
+            for (int v = 0; v < pp.nviews; ++v) a.v[v].E = (uint8_t *)a.v[v].S;
     }
     return a;
 }

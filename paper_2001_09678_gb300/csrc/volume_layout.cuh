@@ -13,4 +13,16 @@ __host__ __device__ __forceinline__ int wide_byte(int k, int nq)
     return l * 4 * nq + (i < 2 * nq ? 2 * i : 2 * (i - 2 * nq) + 1);
 }
 
+// Byte of label k in a 48-label pixel with byte sums: 4 lanes of 12 labels, the lanes' first 8
+// labels, then their last 4.
+__host__ __device__ __forceinline__ int bytes48_of(int k)
+{
+    const int l = k / 12, i = k - l * 12;
+    return i < 8 ? l * 8 + i : 32 + l * 4 + (i - 8);
+}
+__host__ __device__ __forceinline__ int bytes48_label(int b)
+{
+    return b < 32 ? (b >> 3) * 12 + (b & 7) : ((b - 32) >> 2) * 12 + 8 + (b & 3);
+}
+
 }  // namespace mpv
