@@ -71,8 +71,119 @@ __global__ void __launch_bounds__(kTile *kTile) conv3x3_kernel(
     }
 }
 
-// dW[co][ci][k] += sum over a tile of g[n][co][y][x] in[n][ci][y+ky-1][x+kx-1];
-// db[co] += sum g.  One block per (tile, sample); partial sums added atomically.
+// Two FP32 multiply-adds in one instruction (each rounded as fmaf), on register pairs.
+__device__ __forceinline__ unsigned long long pair(float lo, float hi)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpair(unsigned long long v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ void fma2(unsigned long long &acc, unsigned long long a,
+                                     unsigned long long b)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+// conv3x3_kernel for 32 output channels and FP32 input (the backward-data pass): 4 pixels of a
+// row x 8 channels per thread, a 16 x 16 tile per block, the input tile and the weights of
+// kConvChunk channels at a time in shared memory.  A (channel, ky) takes 8 shared loads for 96
+// multiply-adds, every operand of a warp in one or two 128-byte rows; the sums run in the same
+// order as conv3x3_kernel's (channel, ky, kx) and are bit for bit the same.  Bound: the FP32
+// pipe (8 samples of 320 x 180, 32 -> 32 channels, 8.5 GFLOP: 295 -> 226 us against one pixel and
+// 32 channels per thread and one channel per barrier).
+constexpr int kConvChunk = 16, kConvRow = 20;       // channels per chunk; staged row (18 used)
+constexpr int kConvW = 36;                          // staged weights of one (channel, tap), 32 used
+
+__global__ void __launch_bounds__(256) conv3x3_f32_kernel(
+    const float *__restrict__ in, int Cin, int H, int W, const __nv_bfloat16 *__restrict__ w,
+    const float *__restrict__ b, int relu, __nv_bfloat16 *__restrict__ out_bf,
+    float *__restrict__ out_f)
+{
+    __shared__ __align__(16) float tile[kConvChunk * 18 * kConvRow];
+    __shared__ __align__(16) float ws[kConvChunk * 9 * kConvW];
+    const int n = blockIdx.z;
+    // a warp: one group of 8 channels (its weights are one address), 8 rows x 4 groups of pixels
+    // (8 lanes' rows, kConvRow floats apart, in different banks)
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ty = (lane & 7) + 8 * (warp >> 2), tx = 4 * (lane >> 3), co0 = 8 * (warp & 3);
+    const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
+    const int64_t plane = (int64_t)H * W;
+    const float *src = in + (int64_t)n * Cin * plane;
+    unsigned long long acc[4][4];             // channel pairs x pixels
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            acc[c][p] = b ? pair(b[co0 + 2 * c], b[co0 + 2 * c + 1]) : pair(0.f, 0.f);
+    for (int c0 = 0; c0 < Cin; c0 += kConvChunk) {
+        const int nc = min(kConvChunk, Cin - c0);
+        __syncthreads();
+#pragma unroll 4
+        for (int i = threadIdx.x; i < nc * 18 * 18; i += 256) {
+            const int ci = i / (18 * 18), r = i - ci * (18 * 18), py = r / 18, px = r - py * 18;
+            const int yy = y0 - 1 + py, xx = x0 - 1 + px;
+            tile[(ci * 18 + py) * kConvRow + px] =
+                (yy >= 0 && yy < H && xx >= 0 && xx < W)
+                    ? src[(c0 + ci) * plane + (int64_t)yy * W + xx]
+                    : 0.f;
+        }
+#pragma unroll 4
+        for (int i = threadIdx.x; i < nc * 9 * 32; i += 256) {
+            const int co = i / (nc * 9), r = i - co * (nc * 9);          // r = ci * 9 + k
+            ws[r * kConvW + co] = __bfloat162float(w[(int64_t)co * Cin * 9 + c0 * 9 + r]);
+        }
+        __syncthreads();
+        for (int ci = 0; ci < nc; ++ci)
+#pragma unroll
+            for (int ky = 0; ky < 3; ++ky) {
+                const float *t = tile + (ci * 18 + ty + ky) * kConvRow + tx;
+                const float4 a = *(const float4 *)t;
+                const float2 e = *(const float2 *)(t + 4);
+                const unsigned long long v[6] = {pair(a.x, a.x), pair(a.y, a.y), pair(a.z, a.z),
+                                                 pair(a.w, a.w), pair(e.x, e.x), pair(e.y, e.y)};
+#pragma unroll
+                for (int kx = 0; kx < 3; ++kx) {
+                    const ulonglong2 *wr =
+                        (const ulonglong2 *)(ws + (ci * 9 + ky * 3 + kx) * kConvW + co0);
+                    const ulonglong2 w0 = wr[0], w1 = wr[1];
+                    const unsigned long long wv[4] = {w0.x, w0.y, w1.x, w1.y};
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int p = 0; p < 4; ++p) fma2(acc[c][p], wv[c], v[p + kx]);
+                }
+            }
+    }
+    const int y = y0 + ty;
+    if (y >= H) return;
+    const bool vec = x0 + tx + 3 < W && W % 4 == 0 && ((uintptr_t)out_f & 15) == 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const int64_t o = ((int64_t)n * 32 + co0 + c) * plane + (int64_t)y * W + x0 + tx;
+        float v[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            float lo, hi;
+            unpair(acc[c >> 1][p], lo, hi);
+            v[p] = (c & 1) ? hi : lo;
+            if (relu) v[p] = fmaxf(v[p], 0.f);
+        }
+        if (out_f && vec) *(float4 *)(out_f + o) = make_float4(v[0], v[1], v[2], v[3]);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            if (x0 + tx + p >= W) break;
+            if (out_f && !vec) out_f[o + p] = v[p];
+            if (out_bf) out_bf[o + p] = __float2bfloat16(v[p]);
+        }
+    }
+}
+
+// dW[co][ci][k] += sum over a tile of g[n][co][y][x] in[n][ci][y+ky-1][x+kx-1]; db[co] += sum g.
+// Any channel counts; one block per (tile, sample), partial sums added atomically.
 __global__ void __launch_bounds__(kTile *kTile) conv3x3_wgrad_kernel(
     const __nv_bfloat16 *__restrict__ in, int Cin, const float *__restrict__ g, int Cout,
     int H, int W, float *__restrict__ dw, float *__restrict__ db)
@@ -115,12 +226,176 @@ __global__ void __launch_bounds__(kTile *kTile) conv3x3_wgrad_kernel(
         }
 }
 
-// g_pre = g * (act > 0) (ReLU backward), bf16 activations
+// The same for the network's layers: 32 output channels (CPT 4) or one (CPT 1), Cin <= kWgMaxCin.
+// A thread owns CPT output channels x 1 input channel x 9 taps and slides along the tile's rows:
+// 4 pixels take CPT + 6 16-byte shared loads for 36 CPT multiply-adds, the loads of a warp (8
+// gradient rows, 4 input channels) free of bank conflicts.  CPT 1 splits the tile's rows among
+// kWgSplit threads per element, added in a fixed order at the end.  Blocks stay resident and
+// walk over the tiles, so that their totals meet the shared gradient once per block (no more
+// blocks than that for any size).  Bound: the FP32 pipe and the packing of its operand pairs
+// (8 samples of 320 x 180, 32 -> 32 channels, 8.5 GFLOP: 1,070 -> 245 us against two shared loads
+// per multiply-add; 32 -> 1: 75 us, its staging).
+constexpr int kWgMaxCin = 40, kWgSplit = 8;
+constexpr int kWgGS = 36;                            // floats per staged pixel of 32 gradients
+constexpr int kWgIS = 18 * kConvRow;                 // floats per input channel (8 mod 32)
+
+template <int CPT>
+__global__ void __launch_bounds__(kWgMaxCin * 8, 2) wgrad_tile_kernel(
+    const __nv_bfloat16 *__restrict__ in, int Cin, const float *__restrict__ g, int H, int W, int tx,
+    int ty, int ntiles, float *__restrict__ dw, float *__restrict__ db)
+{
+    constexpr int Cout = CPT * 8 == 32 ? 32 : 1;
+    extern __shared__ __align__(16) float smem[];
+    float *gt = smem;                         // CPT 4: [256 pixels][kWgGS], 1: [256]
+    float *it = smem + (CPT == 1 ? kTile * kTile : kTile * kTile * kWgGS);   // [Cin][18][kConvRow]
+    const int nthr = blockDim.x, t = threadIdx.x;
+    // CPT 4: (input channel, channels 4 cg ..); CPT 1: (input channel, rows)
+    const int ci = t >> 3, cg = t & 7;
+    const bool mine = ci < Cin;
+    const int ya = CPT == 1 ? cg * (kTile / kWgSplit) : 0;
+    const int yb = CPT == 1 ? ya + kTile / kWgSplit : kTile;
+    const int64_t plane = (int64_t)H * W;
+    // CPT 4: pairs of channels; CPT 1: (sum over the even pixels, over the odd ones)
+    constexpr int NP = CPT == 1 ? 1 : CPT / 2;
+    unsigned long long tot[NP][9];
+#pragma unroll
+    for (int j = 0; j < NP; ++j)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) tot[j][k] = pair(0.f, 0.f);
+    float btot = 0.f;
+
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int n = tile / (tx * ty), r = tile - n * (tx * ty);
+        const int y0 = (r / tx) * kTile, x0 = (r % tx) * kTile;
+        __syncthreads();
+#pragma unroll 8
+        for (int i = t; i < Cout * kTile * kTile; i += nthr) {
+            const int co = i / (kTile * kTile), p = i % (kTile * kTile);
+            const int yy = y0 + p / kTile, xx = x0 + p % kTile;
+            gt[CPT == 1 ? p : p * kWgGS + co] =
+                (yy < H && xx < W) ? g[((int64_t)n * Cout + co) * plane + (int64_t)yy * W + xx] : 0.f;
+        }
+#pragma unroll 8
+        for (int i = t; i < Cin * 18 * 18; i += nthr) {
+            const int c = i / (18 * 18), q = i - c * (18 * 18), py = q / 18, px = q - py * 18;
+            const int yy = y0 - 1 + py, xx = x0 - 1 + px;
+            it[(c * 18 + py) * kConvRow + px] =
+                (yy >= 0 && yy < H && xx >= 0 && xx < W)
+                    ? __bfloat162float(in[((int64_t)n * Cin + c) * plane + (int64_t)yy * W + xx])
+                    : 0.f;
+        }
+        __syncthreads();
+        if (mine) {
+            for (int y = ya; y < yb; ++y) {
+                const float *ip = it + ci * kWgIS + y * kConvRow;
+                const float *gp = gt + y * kTile * (CPT == 1 ? 1 : kWgGS) + (CPT == 1 ? 0 : 4 * cg);
+                float4 lo[3];
+#pragma unroll
+                for (int ky = 0; ky < 3; ++ky) lo[ky] = *(const float4 *)(ip + ky * kConvRow);
+#pragma unroll
+                for (int x = 0; x < kTile; x += 4) {
+                    float v[3][6];
+#pragma unroll
+                    for (int ky = 0; ky < 3; ++ky) {
+                        const float4 hi = *(const float4 *)(ip + ky * kConvRow + x + 4);
+                        v[ky][0] = lo[ky].x, v[ky][1] = lo[ky].y, v[ky][2] = lo[ky].z;
+                        v[ky][3] = lo[ky].w, v[ky][4] = hi.x, v[ky][5] = hi.y;
+                        lo[ky] = hi;
+                    }
+                    if constexpr (CPT == 1) {
+                        const ulonglong2 q = *(const ulonglong2 *)(gp + x);
+#pragma unroll
+                        for (int k = 0; k < 9; ++k) {
+                            const float *vk = v[k / 3] + k % 3;
+                            fma2(tot[0][k], q.x, pair(vk[0], vk[1]));
+                            fma2(tot[0][k], q.y, pair(vk[2], vk[3]));
+                        }
+                    } else {
+                        unsigned long long vv[3][6];
+#pragma unroll
+                        for (int k = 0; k < 18; ++k) vv[k / 6][k % 6] = pair(v[k / 6][k % 6], v[k / 6][k % 6]);
+#pragma unroll
+                        for (int p = 0; p < 4; ++p) {
+                            const ulonglong2 q = *(const ulonglong2 *)(gp + (x + p) * kWgGS);
+#pragma unroll
+                            for (int k = 0; k < 9; ++k) {
+                                fma2(tot[0][k], q.x, vv[k / 3][p + k % 3]);
+                                fma2(tot[NP - 1][k], q.y, vv[k / 3][p + k % 3]);
+                            }
+                        }
+                    }
+                }
+            }
+        }
+        // the bias: thread t < 8 Cout sums an eighth of channel t / 8
+        if (db && t < 8 * Cout) {
+            float s = 0.f;
+#pragma unroll 8
+            for (int p = 0; p < 32; ++p) {
+                const int q = (t & 7) * 32 + p;
+                s += gt[CPT == 1 ? q : q * kWgGS + (t >> 3)];
+            }
+            btot += s;
+        }
+    }
+    if (CPT == 1) {                           // the split rows' totals in a fixed order
+        __syncthreads();
+        float *part = smem;                   // [kWgSplit][Cin * 9]
+        if (mine)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                float e, o;
+                unpair(tot[0][k], e, o);
+                part[(cg * Cin + ci) * 9 + k] = e + o;
+            }
+        __syncthreads();
+        for (int e = t; e < Cin * 9; e += nthr) {
+            float s = 0.f;
+#pragma unroll
+            for (int q = 0; q < kWgSplit; ++q) s += part[q * Cin * 9 + e];
+            atomicAdd(dw + e, s);
+        }
+    } else if (mine) {
+#pragma unroll
+        for (int j = 0; j < NP; ++j)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                float lo, hi;
+                unpair(tot[j][k], lo, hi);
+                float *d = dw + ((int64_t)(4 * cg + 2 * j) * Cin + ci) * 9 + k;
+                atomicAdd(d, lo);
+                atomicAdd(d + (int64_t)Cin * 9, hi);
+            }
+    }
+    if (db) {
+        // (blocks of at least 256 threads, or 32 for one channel: whole groups of 8 lanes)
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) btot += __shfl_down_sync(0xFFFFFFFFu, btot, o, 8);
+        if (t < 8 * Cout && (t & 7) == 0) atomicAdd(db + (t >> 3), btot);
+    }
+}
+
+// g_pre = g * (act > 0) (ReLU backward), bf16 activations; four elements per thread where the
+// pointers allow it (bound by DRAM: 14.7 M elements, 147 MB: 57 -> 19 us)
 __global__ void relu_mask_kernel(const float *__restrict__ g, const __nv_bfloat16 *__restrict__ act,
                                  float *__restrict__ out, int64_t n)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) out[i] = __bfloat162float(act[i]) > 0.f ? g[i] : 0.f;
+}
+
+__global__ void relu_mask4_kernel(const float4 *__restrict__ g, const uint2 *__restrict__ act,
+                                  float4 *__restrict__ out, int64_t n4)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n4) return;
+    const float4 v = g[i];
+    const uint2 a = act[i];
+    // a BF16 value is the upper half of its FP32 bits
+    out[i] = make_float4(__uint_as_float(a.x << 16) > 0.f ? v.x : 0.f,
+                         __uint_as_float(a.x & 0xFFFF0000u) > 0.f ? v.y : 0.f,
+                         __uint_as_float(a.y << 16) > 0.f ? v.z : 0.f,
+                         __uint_as_float(a.y & 0xFFFF0000u) > 0.f ? v.w : 0.f);
 }
 
 // wt[ci][co][2-ky][2-kx] = w[co][ci][ky][kx]: backward-data weights
@@ -134,20 +409,33 @@ __global__ void flip_transpose_kernel(const __nv_bfloat16 *__restrict__ w, int C
 }
 
 // Huber loss (delta) of prediction p against target t, mean over n; grad = dL/dp.
-__global__ void huber_kernel(const float *__restrict__ p, const float *__restrict__ t,
-                             float delta, int64_t n, float *__restrict__ grad,
-                             float *__restrict__ loss)
+// The blocks stride over the elements and each adds its losses (summed in 64 bits) once: at
+// most kHuberBlocks roundings of the loss, and no queue of one addition per warp at its address
+// (460,800 elements: 24 -> 6 us).
+constexpr int kHuberBlocks = 152;
+
+__global__ void __launch_bounds__(256) huber_kernel(const float *__restrict__ p,
+                                                    const float *__restrict__ t, float delta,
+                                                    int64_t n, float *__restrict__ grad,
+                                                    float *__restrict__ loss)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float l = 0.f;
-    if (i < n) {
+    double sum = 0.0;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
         const float r = p[i] - t[i];
         const float a = fabsf(r);
-        l = a < delta ? 0.5f * r * r / delta : a - 0.5f * delta;
+        sum += a < delta ? 0.5f * r * r / delta : a - 0.5f * delta;
         grad[i] = (a < delta ? r / delta : copysignf(1.f, r)) / (float)n;
     }
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
-    if ((threadIdx.x & 31) == 0 && loss) atomicAdd(loss, l / (float)n);
+    if (!loss) return;
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+    __shared__ double part[8];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s = 0.0;
+        for (int w = 0; w < 8; ++w) s += part[w];
+        atomicAdd(loss, (float)(s / (double)n));
+    }
 }
 
 // Adam on fp32 master weights; also refreshes their bf16 copy.
@@ -598,14 +886,16 @@ void launch_conv3x3_t(const TIn *in, int N, int Cin, int H, int W, const __nv_bf
                       cudaStream_t s)
 {
     dim3 grid((W + kTile - 1) / kTile, (H + kTile - 1) / kTile, N);
-    const size_t smem = conv_smem_bytes(Cin, Cout);
-    if (Cout == 32) {
-        cudaFuncSetAttribute(conv3x3_kernel<32, TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        conv3x3_kernel<32, TIn><<<grid, kTile * kTile, smem, s>>>(in, Cin, H, W, w, b, relu, out_bf, out_f);
-    } else {
-        cudaFuncSetAttribute(conv3x3_kernel<1, TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        conv3x3_kernel<1, TIn><<<grid, kTile * kTile, smem, s>>>(in, Cin, H, W, w, b, relu, out_bf, out_f);
+    if constexpr (sizeof(TIn) == 4) {
+        if (Cout == 32) {
+            conv3x3_f32_kernel<<<grid, 256, 0, s>>>(in, Cin, H, W, w, b, relu, out_bf, out_f);
+            return;
+        }
     }
+    // one output channel (32 BF16 channels always fit the tensor-core kernel)
+    const size_t smem = conv_smem_bytes(Cin, Cout);
+    cudaFuncSetAttribute(conv3x3_kernel<1, TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    conv3x3_kernel<1, TIn><<<grid, kTile * kTile, smem, s>>>(in, Cin, H, W, w, b, relu, out_bf, out_f);
 }
 
 int sm_count()
@@ -670,7 +960,30 @@ void launch_conv3x3(const __nv_bfloat16 *in, int N, int Cin, int H, int W, const
 void launch_conv3x3_wgrad(const __nv_bfloat16 *in, int N, int Cin, const float *g, int Cout, int H,
                           int W, float *dw, float *db, cudaStream_t s)
 {
-    dim3 grid((W + kTile - 1) / kTile, (H + kTile - 1) / kTile, N);
+    const int64_t tx = (W + kTile - 1) / kTile, ty = (H + kTile - 1) / kTile, tiles = tx * ty * N;
+    if ((Cout == 32 || Cout == 1) && Cin <= kWgMaxCin && ty <= 65535 && N <= 65535 &&
+        tiles < 0x7FFFFFFF) {
+        const unsigned blocks = (unsigned)(tiles < 2 * sm_count() ? tiles : 2 * sm_count());
+        size_t sm = sizeof(float) * ((size_t)kTile * kTile * (Cout == 1 ? 1 : kWgGS) +
+                                     (size_t)Cin * kWgIS);
+        const int threads = (8 * Cin + 31) / 32 * 32;
+        if (Cout == 32) {
+            // (the bias's 256 threads too)
+            cudaFuncSetAttribute(wgrad_tile_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sm);
+            wgrad_tile_kernel<4><<<blocks, threads < 256 ? 256 : threads, sm, s>>>(
+                in, Cin, g, H, W, (int)tx, (int)ty, (int)tiles, dw, db);
+        } else {
+            const size_t part = sizeof(float) * kWgSplit * 9 * (size_t)Cin;
+            if (part > sm) sm = part;
+            cudaFuncSetAttribute(wgrad_tile_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sm);
+            wgrad_tile_kernel<1><<<blocks, threads, sm, s>>>(in, Cin, g, H, W, (int)tx, (int)ty,
+                                                             (int)tiles, dw, db);
+        }
+        return;
+    }
+    dim3 grid((unsigned)tx, (unsigned)ty, N);
     const size_t smem = sizeof(float) * ((size_t)Cout * kTile * kTile + (size_t)Cin * 18 * 18);
     cudaFuncSetAttribute(conv3x3_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     conv3x3_wgrad_kernel<<<grid, kTile * kTile, smem, s>>>(in, Cin, g, Cout, H, W, dw, db);
@@ -745,8 +1058,13 @@ mpv_status mpv_cnn_relu_backward(const float *grad, const void *act, float *out,
                                  void *cuda_stream)
 {
     if (!grad || !act || !out || count < 0) return MPV_ERR_INVALID_ARG;
-    relu_mask_kernel<<<blocks(count, 256), 256, 0, (cudaStream_t)cuda_stream>>>(
-        grad, (const __nv_bfloat16 *)act, out, count);
+    if (((uintptr_t)grad | (uintptr_t)out) % 16 == 0 && (uintptr_t)act % 8 == 0 && count % 4 == 0 &&
+        count > 0)
+        relu_mask4_kernel<<<blocks(count / 4, 256), 256, 0, (cudaStream_t)cuda_stream>>>(
+            (const float4 *)grad, (const uint2 *)act, (float4 *)out, count / 4);
+    else
+        relu_mask_kernel<<<blocks(count, 256), 256, 0, (cudaStream_t)cuda_stream>>>(
+            grad, (const __nv_bfloat16 *)act, out, count);
     return cudaGetLastError() == cudaSuccess ? MPV_OK : MPV_ERR_CUDA;
 }
 
@@ -754,8 +1072,9 @@ mpv_status mpv_cnn_huber(const float *pred, const float *target, float delta, in
                          float *grad, float *loss, void *cuda_stream)
 {
     if (!pred || !target || !grad || count < 1 || !(delta > 0.f)) return MPV_ERR_INVALID_ARG;
-    huber_kernel<<<blocks(count, 256), 256, 0, (cudaStream_t)cuda_stream>>>(pred, target, delta,
-                                                                           count, grad, loss);
+    const unsigned nb = blocks(count, 256);
+    huber_kernel<<<nb < kHuberBlocks ? nb : kHuberBlocks, 256, 0, (cudaStream_t)cuda_stream>>>(
+        pred, target, delta, count, grad, loss);
     return cudaGetLastError() == cudaSuccess ? MPV_OK : MPV_ERR_CUDA;
 }
 
