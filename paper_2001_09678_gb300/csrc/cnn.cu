@@ -93,7 +93,7 @@ __device__ __forceinline__ void fma2(unsigned long long &acc, unsigned long long
 // kConvChunk channels at a time in shared memory.  A (channel, ky) takes 8 shared loads for 96
 // multiply-adds, every operand of a warp in one or two 128-byte rows; the sums run in the same
 // order as conv3x3_kernel's (channel, ky, kx) and are bit for bit the same.  Bound: the FP32
-// pipe (8 samples of 320 x 180, 32 -> 32 channels, 8.5 GFLOP: 295 -> 226 us against one pixel and
+// pipe (8 samples of 320 x 180, 32 -> 32 channels, 8.5 GFLOP: 295 -> 183 us against one pixel and
 // 32 channels per thread and one channel per barrier).
 constexpr int kConvChunk = 16, kConvRow = 20;       // channels per chunk; staged row (18 used)
 constexpr int kConvW = 36;                          // staged weights of one (channel, tap), 32 used
@@ -122,19 +122,23 @@ __global__ void __launch_bounds__(256) conv3x3_f32_kernel(
     for (int c0 = 0; c0 < Cin; c0 += kConvChunk) {
         const int nc = min(kConvChunk, Cin - c0);
         __syncthreads();
-#pragma unroll 4
-        for (int i = threadIdx.x; i < nc * 18 * 18; i += 256) {
-            const int ci = i / (18 * 18), r = i - ci * (18 * 18), py = r / 18, px = r - py * 18;
-            const int yy = y0 - 1 + py, xx = x0 - 1 + px;
-            tile[(ci * 18 + py) * kConvRow + px] =
-                (yy >= 0 && yy < H && xx >= 0 && xx < W)
-                    ? src[(c0 + ci) * plane + (int64_t)yy * W + xx]
-                    : 0.f;
+        // a thread keeps its pixels and walks over the channels
+        for (int i = threadIdx.x; i < 18 * 18; i += 256) {
+            const int py = i / 18, px = i - py * 18, yy = y0 - 1 + py, xx = x0 - 1 + px;
+            const bool in_map = yy >= 0 && yy < H && xx >= 0 && xx < W;
+            const float *p = src + (c0 * plane + (int64_t)yy * W + xx);
+            float v[kConvChunk];
+#pragma unroll
+            for (int c = 0; c < kConvChunk; ++c) v[c] = in_map && c < nc ? p[c * plane] : 0.f;
+#pragma unroll
+            for (int c = 0; c < kConvChunk; ++c) tile[(c * 18 + py) * kConvRow + px] = v[c];
         }
-#pragma unroll 4
-        for (int i = threadIdx.x; i < nc * 9 * 32; i += 256) {
-            const int co = i / (nc * 9), r = i - co * (nc * 9);          // r = ci * 9 + k
-            ws[r * kConvW + co] = __bfloat162float(w[(int64_t)co * Cin * 9 + c0 * 9 + r]);
+        {
+            const int co = threadIdx.x >> 3;
+            const __nv_bfloat16 *p = w + (int64_t)co * Cin * 9 + c0 * 9;
+#pragma unroll 9
+            for (int r = threadIdx.x & 7; r < nc * 9; r += 8)               // r = ci * 9 + k
+                ws[r * kConvW + co] = __bfloat162float(p[r]);
         }
         __syncthreads();
         for (int ci = 0; ci < nc; ++ci)
@@ -229,18 +233,19 @@ __global__ void __launch_bounds__(kTile *kTile) conv3x3_wgrad_kernel(
 // The same for the network's layers: 32 output channels (CPT 4) or one (CPT 1), Cin <= kWgMaxCin.
 // A thread owns CPT output channels x 1 input channel x 9 taps and slides along the tile's rows:
 // 4 pixels take CPT + 6 16-byte shared loads for 36 CPT multiply-adds, the loads of a warp (8
-// gradient rows, 4 input channels) free of bank conflicts.  CPT 1 splits the tile's rows among
-// kWgSplit threads per element, added in a fixed order at the end.  Blocks stay resident and
-// walk over the tiles, so that their totals meet the shared gradient once per block (no more
-// blocks than that for any size).  Bound: the FP32 pipe and the packing of its operand pairs
-// (8 samples of 320 x 180, 32 -> 32 channels, 8.5 GFLOP: 1,070 -> 245 us against two shared loads
-// per multiply-add; 32 -> 1: 75 us, its staging).
+// gradient groups, or 8 rows, and 4 input channels) free of bank conflicts.  CPT 1 splits the
+// tile's rows among kWgSplit threads per element, added in a fixed order at the end.  Blocks
+// stay resident and walk over the tiles, so that their totals meet the shared gradient once per
+// block.  Bound: the FP32 pipe and the packing of its operand pairs (8 samples of 320 x 180,
+// 32 -> 32 channels, 8.5 GFLOP: 1,070 -> 220 us against two shared loads per multiply-add;
+// 32 -> 1: 59 us, its staging).  Staging by an element's index, with its divisions, instead of
+// a thread's fixed pixels: 245 us.
 constexpr int kWgMaxCin = 40, kWgSplit = 8;
 constexpr int kWgGS = 36;                            // floats per staged pixel of 32 gradients
 constexpr int kWgIS = 18 * kConvRow;                 // floats per input channel (8 mod 32)
 
 template <int CPT>
-__global__ void __launch_bounds__(kWgMaxCin * 8, 2) wgrad_tile_kernel(
+__global__ void __launch_bounds__(kWgMaxCin * 8, CPT == 1 ? 3 : 2) wgrad_tile_kernel(
     const __nv_bfloat16 *__restrict__ in, int Cin, const float *__restrict__ g, int H, int W, int tx,
     int ty, int ntiles, float *__restrict__ dw, float *__restrict__ db)
 {
@@ -252,8 +257,7 @@ __global__ void __launch_bounds__(kWgMaxCin * 8, 2) wgrad_tile_kernel(
     // CPT 4: (input channel, channels 4 cg ..); CPT 1: (input channel, rows)
     const int ci = t >> 3, cg = t & 7;
     const bool mine = ci < Cin;
-    const int ya = CPT == 1 ? cg * (kTile / kWgSplit) : 0;
-    const int yb = CPT == 1 ? ya + kTile / kWgSplit : kTile;
+    const int ya = CPT == 1 ? cg : 0, ystep = CPT == 1 ? kWgSplit : 1;
     const int64_t plane = (int64_t)H * W;
     // CPT 4: pairs of channels; CPT 1: (sum over the even pixels, over the odd ones)
     constexpr int NP = CPT == 1 ? 1 : CPT / 2;
@@ -268,25 +272,44 @@ __global__ void __launch_bounds__(kWgMaxCin * 8, 2) wgrad_tile_kernel(
         const int n = tile / (tx * ty), r = tile - n * (tx * ty);
         const int y0 = (r / tx) * kTile, x0 = (r % tx) * kTile;
         __syncthreads();
-#pragma unroll 8
-        for (int i = t; i < Cout * kTile * kTile; i += nthr) {
-            const int co = i / (kTile * kTile), p = i % (kTile * kTile);
-            const int yy = y0 + p / kTile, xx = x0 + p % kTile;
-            gt[CPT == 1 ? p : p * kWgGS + co] =
-                (yy < H && xx < W) ? g[((int64_t)n * Cout + co) * plane + (int64_t)yy * W + xx] : 0.f;
+        // a thread keeps its pixels and walks over the channels
+        for (int i = t; i < kTile * kTile; i += nthr) {
+            const int yy = y0 + i / kTile, xx = x0 + i % kTile;
+            const bool in_map = yy < H && xx < W;
+            const float *p = g + ((int64_t)n * Cout * plane + (int64_t)yy * W + xx);
+            if (CPT == 1) {
+                gt[i] = in_map ? *p : 0.f;
+            } else {
+#pragma unroll
+                for (int c = 0; c < Cout; c += 16) {
+                    float v[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] = in_map ? p[(c + j) * plane] : 0.f;
+#pragma unroll
+                    for (int j = 0; j < 16; j += 4)
+                        *(float4 *)(gt + i * kWgGS + c + j) =
+                            make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                }
+            }
         }
-#pragma unroll 8
-        for (int i = t; i < Cin * 18 * 18; i += nthr) {
-            const int c = i / (18 * 18), q = i - c * (18 * 18), py = q / 18, px = q - py * 18;
-            const int yy = y0 - 1 + py, xx = x0 - 1 + px;
-            it[(c * 18 + py) * kConvRow + px] =
-                (yy >= 0 && yy < H && xx >= 0 && xx < W)
-                    ? __bfloat162float(in[((int64_t)n * Cin + c) * plane + (int64_t)yy * W + xx])
-                    : 0.f;
+        for (int i = t; i < 18 * 18; i += nthr) {
+            const int py = i / 18, px = i - py * 18, yy = y0 - 1 + py, xx = x0 - 1 + px;
+            const bool in_map = yy >= 0 && yy < H && xx >= 0 && xx < W;
+            const __nv_bfloat16 *p = in + ((int64_t)n * Cin * plane + (int64_t)yy * W + xx);
+            float *d = it + py * kConvRow + px;
+            for (int c = 0; c < Cin; c += 8, p += 8 * plane, d += 8 * kWgIS) {
+                float v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    v[j] = in_map && c + j < Cin ? __bfloat162float(p[j * plane]) : 0.f;
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (c + j < Cin) d[j * kWgIS] = v[j];
+            }
         }
         __syncthreads();
         if (mine) {
-            for (int y = ya; y < yb; ++y) {
+            for (int y = ya; y < kTile; y += ystep) {
                 const float *ip = it + ci * kWgIS + y * kConvRow;
                 const float *gp = gt + y * kTile * (CPT == 1 ? 1 : kWgGS) + (CPT == 1 ? 0 : 4 * cg);
                 float4 lo[3];
@@ -963,7 +986,8 @@ void launch_conv3x3_wgrad(const __nv_bfloat16 *in, int N, int Cin, const float *
     const int64_t tx = (W + kTile - 1) / kTile, ty = (H + kTile - 1) / kTile, tiles = tx * ty * N;
     if ((Cout == 32 || Cout == 1) && Cin <= kWgMaxCin && ty <= 65535 && N <= 65535 &&
         tiles < 0x7FFFFFFF) {
-        const unsigned blocks = (unsigned)(tiles < 2 * sm_count() ? tiles : 2 * sm_count());
+        const int64_t resident = (Cout == 1 ? 3 : 2) * (int64_t)sm_count();
+        const unsigned blocks = (unsigned)(tiles < resident ? tiles : resident);
         size_t sm = sizeof(float) * ((size_t)kTile * kTile * (Cout == 1 ? 1 : kWgGS) +
                                      (size_t)Cin * kWgIS);
         const int threads = (8 * Cin + 31) / 32 * 32;
