@@ -37,10 +37,7 @@
 //  * agg_general: any window width: one warp per scan path, the sweeps written as prefix
 //    minima  min_{v<=u} A(v) + p1 (u-v) = p1 u + min_{v<=u} (A(v) - p1 v)  (and the mirror
 //    image), evaluated by shuffle scans over the lanes.
-#define MIN3 1
-#ifndef MIXDYN
-#define MIXDYN 0
-#endif
+#include "agg_layer.cuh"
 #include "agg_rows.cuh"
 
 namespace mpv {
@@ -777,20 +774,35 @@ template <int G, int KW>
 void launch_layer_kw(const LevelArgs &a, const MergeArgs &m, cudaStream_t s)
 {
     const bool win = a.v[0].lo != nullptr;
-    const bool blk = a.block_cut > 0;
-    if (a.radius <= 2) {
-        if (win) launch_stencil<G, KW, 2, true, false, true, false, G == 8>(a, s, m, m.ndirs);
-        else if (blk) launch_stencil<G, KW, 2, false, true, true, false, G == 8>(a, s, m, m.ndirs);
-        else launch_stencil<G, KW, 2, false, false, true, false, G == 8>(a, s, m, m.ndirs);
-    } else if constexpr (KW >= 2) {
+    if constexpr (G == 8 && KW >= 1) {
+        if (a.radius <= 2) {       // (with tiles only: agg_layer takes the rest)
+            launch_stencil<G, KW, 2, false, true, true, false, true>(a, s, m, m.ndirs);
+            return;
+        }
+    }
+    if constexpr (KW >= 2) {
         if (win) launch_stencil<G, KW, 4, true, false, true, false, G == 8>(a, s, m, m.ndirs);
-        else if (blk) launch_stencil<G, KW, 4, false, true, true, false, G == 8>(a, s, m, m.ndirs);
+        else if (a.block_cut > 0)
+            launch_stencil<G, KW, 4, false, true, true, false, G == 8>(a, s, m, m.ndirs);
         else launch_stencil<G, KW, 4, false, false, true, false, G == 8>(a, s, m, m.ndirs);
     }
 }
 
+// Radius at most 2 without tiles runs on agg_layer (its steps read staged data only; both
+// shapes and every data term faster than the packed stencil's layer mode, see there).
 void launch_layer_stencil(const LevelArgs &a, const MergeArgs &m, cudaStream_t s)
 {
+    const bool win = a.v[0].lo != nullptr;
+    if (a.radius <= 2 && a.block_cut == 0) {
+        if (a.Dws == 32) {
+            if (win) launch_agg_layer<2, true>(a, m, s);
+            else launch_agg_layer<2, false>(a, m, s);
+        } else {
+            if (win) launch_agg_layer<1, true>(a, m, s);
+            else launch_agg_layer<1, false>(a, m, s);
+        }
+        return;
+    }
     if (a.Dws == 32) launch_layer_kw<kLanesWide, 2>(a, m, s);
     else if (a.radius <= 2) launch_layer_kw<kLanesWide, 1>(a, m, s);
     else launch_layer_kw<4, 2>(a, m, s);
