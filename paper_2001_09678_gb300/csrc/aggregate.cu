@@ -39,6 +39,7 @@
 //    image), evaluated by shuffle scans over the lanes.
 #include "agg_layer.cuh"
 #include "agg_rows.cuh"
+#include "agg_sweep.cuh"
 
 namespace mpv {
 
@@ -916,6 +917,20 @@ bool bytes_ok(const LevelArgs &a)
 {
     return a.radius <= 2 && a.Dws <= 64 && a.block_cut == 0 &&
            (int64_t)a.npaths * a.trunc <= 255 && packed_caps_ok(a, 1);
+}
+
+// Byte sums of the gradient-weighted passes: strides of 16 and 32 labels, sums that fit a byte, no
+// tiles.  (T <= 63: the continuations of agg_sweep.cuh stay below 2^16.)
+bool sweep_bytes_ok(const LevelArgs &a)
+{
+    return (a.Dws == 16 || a.Dws == 32) && a.block_cut == 0 && a.trunc <= 63 &&
+           (int64_t)a.npaths * a.trunc <= 255;
+}
+
+void launch_sweep_bytes(const LevelArgs &a, const int *lut, cudaStream_t s)
+{
+    if (a.Dws == 16) launch_agg_sweep<2>(a, lut, s);
+    else launch_agg_sweep<4>(a, lut, s);
 }
 
 void launch_aggregate(const LevelArgs &a, cudaStream_t s)

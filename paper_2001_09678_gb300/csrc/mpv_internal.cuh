@@ -133,6 +133,8 @@ void launch_cost(const LevelArgs &a, cudaStream_t s);
 void launch_aggregate(const LevelArgs &a, cudaStream_t s);
 // Whether the summed passes of a level without windows run on wide volumes, and their shape.
 bool bytes_ok(const LevelArgs &a);   // byte sums of the packed stencil apply
+bool sweep_bytes_ok(const LevelArgs &a);   // byte sums of the gradient-weighted passes apply
+void launch_sweep_bytes(const LevelArgs &a, const int *lut, cudaStream_t s);
 bool wide_shape(const LevelArgs &a, int &G, int &NQ);
 void launch_wide(const LevelArgs &a, cudaStream_t s);
 
@@ -299,9 +301,11 @@ struct PairPlan {
 void plan_pair(const mpv_params &p, const PairJob &job, uint8_t *base, int nviews,
                bool level_volumes, PairPlan &pp);
 // Arguments of level l (both views) and of its window seeding (l > 0).
-// sums: the level may use byte sums (summed merge without a gradient table).
+// sums: the byte sums that the level may use (summed merge with one slope, or with the gradient
+// table's).
+enum Sums { kSums16, kSumsBytes, kSumsSweep };
 LevelArgs level_args(const mpv_params &p, const PairPlan &pp, uint8_t *base, int l,
-                     const Tuning &tune, const int *gate, bool sums = false);
+                     const Tuning &tune, const int *gate, Sums sums = kSums16);
 SeedArgs seed_args(const PairPlan &pp, uint8_t *base, int l, const int *gate,
                    int *err = nullptr);
 

@@ -284,7 +284,7 @@ void plan_pair(const mpv_params &p, const PairJob &job, uint8_t *base, int nview
 }
 
 LevelArgs level_args(const mpv_params &p, const PairPlan &pp, uint8_t *base, int l,
-                     const Tuning &tune, const int *gate, bool sums)
+                     const Tuning &tune, const int *gate, Sums sums)
 {
     const Geometry &g = pp.g;
     const Layout &L = pp.L;
@@ -323,14 +323,14 @@ LevelArgs level_args(const mpv_params &p, const PairPlan &pp, uint8_t *base, int
         vl.S2 = nullptr;
         vl.E = nullptr;
     }
-    if (sums && l == 0 && wide_shape(a, a.wide_g, a.wide_nq)) {
+    if (sums == kSumsBytes && l == 0 && wide_shape(a, a.wide_g, a.wide_nq)) {
         // C and E share the region of C and S (adjacent, 3 Dws bytes per pixel, no fewer than
         // two wide volumes); E starts on 8 bytes
         const size_t vol = (size_t)a.W * a.H * (4 * a.wide_g * a.wide_nq);
         for (int v = 0; v < pp.nviews; ++v) a.v[v].E = a.v[v].C + vol;
     } else {
         a.wide_g = a.wide_nq = 0;
-        a.bytes = sums && bytes_ok(a);
+        a.bytes = sums == kSumsBytes ? bytes_ok(a) : (sums == kSumsSweep && sweep_bytes_ok(a));
         if (a.bytes)
             for (int v = 0; v < pp.nviews; ++v) a.v[v].E = (uint8_t *)a.v[v].S;
     }
@@ -446,7 +446,9 @@ mpv_status enqueue_pair(const mpv_params &p, const PairJob &job, uint8_t *base, 
     for (int l = 0; l <= last; ++l) {
         if (learned && l > 0 && l < top) continue;
         // (the network's features read the top level's plain volume)
-        const bool sums = !layered && !grad_lut && !(learned && l == 0) && !(dbg && dbg->plain);
+        const Sums sums = layered || (learned && l == 0) || (dbg && dbg->plain)
+                              ? kSums16
+                              : (grad_lut ? kSumsSweep : kSumsBytes);
         LevelArgs a = level_args(p, pp, base, l, tune, gate, sums);
         a.edge = (learned && l == top) ? edge : nullptr;
         if (learned && l == top) {
@@ -532,7 +534,9 @@ mpv_status enqueue_pair(const mpv_params &p, const PairJob &job, uint8_t *base, 
         } else {
             HookScope hs(hook, MPV_STAGE_AGGREGATE, 1, s);
             // S was cleared by the cost kernel
-            if (grad_lut) {
+            if (grad_lut && a.bytes) {
+                launch_sweep_bytes(a, grad_lut, s);
+            } else if (grad_lut) {
                 MergeArgs m{};
                 m.in_mode = 0;
                 m.out_mode = 0;
