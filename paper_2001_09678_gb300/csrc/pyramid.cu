@@ -173,8 +173,10 @@ void launch_wide_wta(const LevelArgs &a, cudaStream_t s)
 }
 
 // Winner-take-all on byte sums: S = npaths C + E, ties to the smallest disparity.  TPP threads
-// per pixel, each with the same DWS / TPP bytes of C and of E.  Bound by DRAM and L2
-// (1280x720, 32 labels, both views: 118 MB in 29 us, 4.0 TB/s; 16-bit sums 41 us).
+// per pixel, each with the same DWS / TPP bytes of C and of E.  A chunk of 16 labels is compared
+// in pairs of 16-bit keys, 16 S + position (S <= 8 * 255 + 255).  Bound by DRAM and L2
+// (1280x720, 32 labels, both views, 118 MB: 22 us; with a 32-bit key per label 29 us, 16-bit sums
+// 41 us).
 template <int DWS, int TPP>
 __global__ void __launch_bounds__(256) bytes_wta_kernel(LevelArgs a)
 {
@@ -197,20 +199,29 @@ __global__ void __launch_bounds__(256) bytes_wta_kernel(LevelArgs a)
             qe[k] = pe[k];
         }
         lo = v.lo ? (int)v.lo[i] : 0;
-        const uint32_t np = (uint32_t)a.npaths << 16;
-        const int first = sub * NV * 16;      // (TPP = 1 for 48 labels)
+        const uint32_t np = 16u * (uint32_t)a.npaths;
+        const bool padded = a.Dw < DWS;
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
             const uint32_t wc[4] = {qc[k].x, qc[k].y, qc[k].z, qc[k].w};
             const uint32_t we[4] = {qe[k].x, qe[k].y, qe[k].z, qe[k].w};
+            // byte b's label, in ascending order of b (TPP = 1 for 48 labels)
+            auto label = [&](int b) {
+                return DWS == 48 ? bytes48_label(16 * k + b) : (sub * NV + k) * 16 + b;
+            };
+            uint32_t m = 0xFFFFFFFFu;
 #pragma unroll
-            for (int b = 0; b < 16; ++b) {
-                const uint32_t c = (wc[b >> 2] >> (8 * (b & 3))) & 0xFFu;
-                const uint32_t e = (we[b >> 2] >> (8 * (b & 3))) & 0xFFu;
-                const int u = DWS == 48 ? bytes48_label(16 * k + b) : first + 16 * k + b;
-                const uint32_t key = c * np + ((e << 16) | (uint32_t)u);
-                if (u < a.Dw) best = min(best, key);
+            for (int b = 0; b < 16; b += 2) {
+                const uint32_t sel = (b & 2) ? 0x4342u : 0x4140u;
+                const uint32_t c = __byte_perm(wc[b >> 2], 0u, sel);
+                const uint32_t e = __byte_perm(we[b >> 2], 0u, sel);
+                uint32_t key = c * np + (e * 16u + (uint32_t)(b | ((b + 1) << 16)));
+                if (padded)
+                    key |= (label(b) < a.Dw ? 0u : 0xFFFFu) | (label(b + 1) < a.Dw ? 0u : 0xFFFF0000u);
+                m = __vminu2(m, key);
             }
+            const uint32_t one = min(m & 0xFFFFu, m >> 16);
+            best = min(best, ((one >> 4) << 16) | (uint32_t)label((int)(one & 15u)));
         }
     }
 #pragma unroll
