@@ -118,9 +118,9 @@ def level_geometry():
 
 ALG_NOTE = {
     "cost": "images 2 B/px + cost write 1 B/node (cost stored as uint8: exact, costs <= 255)",
-    "aggregate": "cost read 1 B + summed-energy write 2 B per node, window starts 2 B/px "
-                 "(the survey's B_alg reads a uint16 cost: 2 B + 2 B, reported as "
-                 "frac_at_survey_bytes)",
+    "aggregate": "cost read 1 B + summed-energy write 2 B per node (16-bit sums; byte sums "
+                 "write 1 B), window starts 2 B/px (the survey's B_alg reads a uint16 cost: "
+                 "2 B + 2 B, reported as frac_at_survey_bytes)",
     "wta": "summed-energy read 2 B/node + window starts and map 2 B/px each",
 }
 

@@ -26,8 +26,9 @@
 //    to be resident at once, agg_rows_first starts the row paths (the W-step chains that
 //    bound such levels) ahead of the other directions in one grid.  Its layer mode
 //    runs one layer of the layered merge (Section 3.2), the left-to-right pass with doubled
-//    upward jumps included; its sweep mode runs gradient-weighted slopes (Eq. EU) as
-//    untruncated packed sweeps.
+//    upward jumps included, for radius 3 to 4 and tiles (agg_layer.cuh takes radius 2); its
+//    sweep mode runs gradient-weighted slopes (Eq. EU) as untruncated packed sweeps, in
+//    layers and where the sums need 16 bits (agg_sweep.cuh takes the rest).
 //  * byte sums (launch_bytes): the same passes where the sums of the energies' increments fit
 //    bytes (8 paths: T <= 31) and jumps beyond 2 labels are truncated, the usual case; the
 //    row directions in agg_rows.cuh, wide levels without windows in agg_wide.cu.
