@@ -105,7 +105,8 @@ __device__ __forceinline__ void wide_scan(const LevelArgs &a, const uint8_t *__r
 
     // the lane's elements of a step: lane + 32 k in the order (path, 8-byte element); columns
     // and diagonals have them contiguous in memory
-    const bool last = 32 * NE == 16 * NQ || lane < 16 * NQ - 32 * (NE - 1);
+    const bool last = 32 * NE == 16 * NQ || wide_elem(NQ, lane, NE - 1);
+    auto elem = [&](int k) { return k + 1 < NE || last; };
     unsigned eo[MODE == 0 ? NE : 1];
     bool eact[MODE == 0 ? NE : 1];
     if (MODE == 0) {
@@ -113,7 +114,7 @@ __device__ __forceinline__ void wide_scan(const LevelArgs &a, const uint8_t *__r
         for (int k = 0; k < NE; ++k) {
             const int e = lane + 32 * k, p = e / EPP;
             eo[k % (MODE == 0 ? NE : 1)] = (unsigned)(p * W * R + (e - p * EPP) * 8);
-            eact[k % (MODE == 0 ? NE : 1)] = (k + 1 < NE || last) && c + p < H;
+            eact[k % (MODE == 0 ? NE : 1)] = elem(k) && c + p < H;
         }
     }
     const uint8_t *pc = C + base * R + (MODE == 0 ? 0 : lane * 8);
@@ -127,7 +128,7 @@ __device__ __forceinline__ void wide_scan(const LevelArgs &a, const uint8_t *__r
     // whether element k belongs to a path that is active at first column cc
     auto has = [&](int k, int cc) {
         if (MODE == 0) return eact[k % (MODE == 0 ? NE : 1)];
-        return (k + 1 < NE || last) && (unsigned)(cc + epath(k)) < (unsigned)lim;
+        return elem(k) && (unsigned)(cc + epath(k)) < (unsigned)lim;
     };
     auto at = [&](int k) -> unsigned {
         return MODE == 0 ? eo[k % (MODE == 0 ? NE : 1)] : (unsigned)(k * 256);
@@ -136,8 +137,12 @@ __device__ __forceinline__ void wide_scan(const LevelArgs &a, const uint8_t *__r
     auto fetch = [&](bool more, unsigned stage) {
         if (more) {
 #pragma unroll
-            for (int k = 0; k < NE; ++k)
-                wide_copy8(csm + stage * STEP + k * 256, pc + at(k), has(k, ca));
+            for (int k = 0; k < NE; ++k) {
+                const bool on = has(k, ca);
+                const uint8_t *src = pc + at(k);
+                wide_copy8(csm + stage * STEP + k * 256, src,
+                           on && MPV_IN(a.err, src >= C && src + 8 <= C + (int64_t)W * H * R, 12));
+            }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
         pc += dstep;
@@ -176,7 +181,15 @@ __device__ __forceinline__ void wide_scan(const LevelArgs &a, const uint8_t *__r
     auto flush = [&](unsigned par) {
         const unsigned long long *src = (const unsigned long long *)(ebuf + par * STEP) + lane;
 #pragma unroll
-        for (int k = 0; k < NE; ++k) wide_add8(pe + at(k), src[32 * k], has(k, cp));
+        for (int k = 0; k < NE; ++k) {
+            // (the element itself, not only its reduction: with an odd NQ the last 16 lanes'
+            // would be past the step)
+            unsigned long long v = 0;
+            if (elem(k) && MPV_IN(a.err, lane + 32 * k < 16 * NQ, 13)) v = src[32 * k];
+            const bool on = has(k, cp);
+            uint8_t *dst = pe + at(k);
+            wide_add8(dst, v, on && MPV_IN(a.err, dst >= E && dst + 8 <= E + (int64_t)W * H * R, 14));
+        }
         pe += dstep;
         if (MODE == 2) {
             if (cp + sx > wv - P) pe -= (int64_t)wv * R;

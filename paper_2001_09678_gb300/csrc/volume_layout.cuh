@@ -13,6 +13,13 @@ __host__ __device__ __forceinline__ int wide_byte(int k, int nq)
     return l * 4 * nq + (i < 2 * nq ? 2 * i : 2 * (i - 2 * nq) + 1);
 }
 
+// A step of a warp's scan of wide volumes is 16 nq elements of 8 bytes, lane + 32 k being the
+// lane's k-th: whether there is one (with an odd nq the last 16 lanes have one fewer).
+__host__ __device__ __forceinline__ bool wide_elem(int nq, int lane, int k)
+{
+    return lane + 32 * k < 16 * nq;
+}
+
 // Byte of label k in a 48-label pixel with byte sums: 4 lanes of 12 labels, the lanes' first 8
 // labels, then their last 4.
 __host__ __device__ __forceinline__ int bytes48_of(int k)
