@@ -83,15 +83,20 @@ __device__ __forceinline__ void layer_body(const LevelArgs &a, const MergeArgs &
     const uint8_t *pa = (PAIR ? (const uint8_t *)qa : V.C) + at0;
     const uint8_t *pb = PAIR ? (const uint8_t *)qb + at0 : nullptr;
     const int64_t dpiece = TPI * dpix * LS::VB;
+    [[maybe_unused]] auto in_volume = [&](const uint8_t *p, const uint8_t *vol) {
+        return p >= vol && p + 16 <= vol + (int64_t)W * H * LS::VB;
+    };
     auto issue = [&](int c) {             // chunk c into stage c & 1; pa, pb point at it
         const uint32_t st = sbase + (c & 1) * (4 * LS::PATHB);
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
             const bool on = c * CH + i * TPI + gl / PPS < n;
-            row_copy(st + i * TPI * LS::STEPB, pa, 16, on);
+            row_copy(st + i * TPI * LS::STEPB, pa, 16,
+                     on && MPV_IN(a.err, in_volume(pa, PAIR ? (const uint8_t *)qa : V.C), 18));
             pa += dpiece;
             if (PAIR) {
-                row_copy(st + i * TPI * LS::STEPB + LS::VB, pb, 16, on);
+                row_copy(st + i * TPI * LS::STEPB + LS::VB, pb, 16,
+                         on && MPV_IN(a.err, in_volume(pb, (const uint8_t *)qb), 18));
                 pb += dpiece;
             }
         }
@@ -101,7 +106,8 @@ __device__ __forceinline__ void layer_body(const LevelArgs &a, const MergeArgs &
     const uint16_t *lp = WIN ? V.lo + pix0 + gl * dpix : nullptr;
     int lo_next = 0;
     auto issue_lo = [&](int c) {
-        if (c * CH + gl < n) lo_next = (int)ld_pin_u16(lp);
+        if (c * CH + gl < n && MPV_IN(a.err, lp >= V.lo && lp < V.lo + (int64_t)W * H, 19))
+            lo_next = (int)ld_pin_u16(lp);
         lp += CH * dpix;
     };
 
@@ -143,6 +149,7 @@ __device__ __forceinline__ void layer_body(const LevelArgs &a, const MergeArgs &
         uint32_t v[KW];
 #pragma unroll
         for (int i = 0; i < KW; ++i) v[i] = (A[i] - m2) & ~pad[i];   // per half: A >= m2
+        if (!MPV_IN(a.err, op >= outv && op + K <= outv + (int64_t)W * H * DWP, 20)) return;
         if (KW == 1) *(uint32_t *)op = v[0];
         else *(uint2 *)op = make_uint2(v[0], v[1 % KW]);
     };
@@ -261,9 +268,11 @@ __device__ __forceinline__ void layer_body(const LevelArgs &a, const MergeArgs &
                         if (i < 2 || gl < LS::PADL / 2 - 16) sb[gl + 8 * i] = m2;
                     __syncwarp();
                     uint32_t Sd[KW + 1];
+                    const bool sok =
+                        MPV_IN(a.err, (int)sh.x + 1 >= 0 && (int)sh.x + 1 + gl * KW + KW < LS::PATHW, 4);
                     const uint32_t *pw = sb + gl * KW + sh.x + 1;
 #pragma unroll
-                    for (int i = 0; i <= KW; ++i) Sd[i] = pw[i];
+                    for (int i = 0; i <= KW; ++i) Sd[i] = sok ? pw[i] : INF2;
 #pragma unroll
                     for (int i = 0; i < KW; ++i) SA[i] = __byte_perm(Sd[i], Sd[i + 1], sh.y);
                 }

@@ -82,15 +82,18 @@ __device__ __forceinline__ void row_bytes_body(const LevelArgs &a, int grp, int 
         for (int i = 0; i < NP; ++i) {
             const int e = lane + 32 * i, r = e / PPR, q = e % PPR;
             const int yr = min(4 * grp + r, H - 1), x = x0 + q * 16 / DWP;
-            row_copy(st + r * RS::ROWB + q * 16,
-                     V.C + ((int64_t)yr * W + x0) * DWP + q * 16, 16, x >= 0 && x < W);
+            const int64_t at = ((int64_t)yr * W + x0) * DWP + q * 16;
+            const bool on = x >= 0 && x < W;
+            row_copy(st + r * RS::ROWB + q * 16, V.C + at, 16,
+                     on && MPV_IN(a.err, at >= 0 && at + 16 <= (int64_t)W * H * DWP, 15));
         }
         if (WIN) {                        // 8 window starts: five aligned words hold them
             const int r = lane / 5, k = lane - 5 * r;
             const int yr = min(4 * grp + r, H - 1);
             const int64_t at = ((((int64_t)yr * W + x0) * 2) & ~(int64_t)3) + 4 * k;
+            const bool on = lane < 20 && at >= 0 && at < (int64_t)W * H * 2;
             row_copy(sbase + RS::off_lo + (c & 1) * 128 + r * 32 + 4 * k, (const uint8_t *)V.lo + at,
-                     4, lane < 20 && at >= 0 && at < (int64_t)W * H * 2);
+                     4, on && MPV_IN(a.err, (at & 3) == 0 && r < 4 && 4 * k < 32, 16));
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -223,7 +226,10 @@ __device__ __forceinline__ void row_bytes_body(const LevelArgs &a, int grp, int 
             } else {
                 out = __byte_perm(inc[0], inc[1 % KW], 0x6420);
             }
-            if (adds && u < n) atomicAdd((unsigned int *)(ep + u * DX * DWP), out);
+            uint8_t *dst = ep + u * DX * DWP;
+            if (adds && u < n &&
+                MPV_IN(a.err, dst >= V.E && dst + 4 <= V.E + (int64_t)W * H * DWP, 17))
+                atomicAdd((unsigned int *)dst, out);
         }
         ep += CH * DX * DWP;
         __syncwarp();                 // every lane is done with the stage that is filled next

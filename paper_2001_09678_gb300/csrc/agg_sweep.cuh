@@ -92,13 +92,18 @@ __device__ __forceinline__ void sweep_body(const LevelArgs &a, const int *lut, i
         const uint32_t st = sbase + (c & 1) * (8 * SS::PATHB);
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
-            row_copy(st + i * TPI * DWP, pc, 16, c * CH + i * TPI + gl / PPS < n);
+            const bool on = c * CH + i * TPI + gl / PPS < n;
+            row_copy(st + i * TPI * DWP, pc, 16,
+                     on && MPV_IN(a.err, pc >= V.C && pc + 16 <= V.C + (int64_t)W * H * DWP, 21));
             pc += dpiece;
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-            if (c * CH + 2 * gl + h < n) {
+            if (c * CH + 2 * gl + h < n &&
+                MPV_IN(a.err, ip + h * di >= V.I0 && ip + h * di < V.I0 + (int64_t)V.pitch0 * (H - 1) + W &&
+                                  (!WIN || (lp + h * dpix >= V.lo && lp + h * dpix < V.lo + (int64_t)W * H)),
+                       22)) {
                 if (WIN) lo_n[h] = (int)ld_pin_u16(lp + h * dpix);
                 in_n[h] = (int)ld_pin_u8(ip + h * di);
             }
