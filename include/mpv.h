@@ -355,7 +355,8 @@ void mpv_server_destroy(mpv_server *srv);
  * when in_f32 = 1; cout is 32 or 1; out_bf16 and/or out_f32 receive the result.
  * BF16 input runs on the tensor cores (tcgen05, FP32 accumulation) while the operands
  * fit in shared memory (cin up to 208); its one device wait is bounded, and outputs of
- * tiles whose wait ran out are NaN.  Larger cin and FP32 input run on the CUDA cores.  */
+ * tiles whose wait ran out are NaN.  FP32 input, and one output channel of larger cin, run
+ * on the CUDA cores.                                                                   */
 mpv_status mpv_cnn_conv3x3(const void *in, int32_t in_f32, int32_t n, int32_t cin, int32_t h,
                            int32_t w, const void *weight, const float *bias, int32_t cout,
                            int32_t relu, void *out_bf16, float *out_f32, void *cuda_stream);

@@ -838,7 +838,7 @@ namespace {
 // lanes for the rows too 308 us; fewer resident blocks (2 to 4 per SM) slower.
 template <int G, int KW, bool WIN, bool PD>
 __global__ void __launch_bounds__(kStencilWarps * 32) agg_mixed(LevelArgs a, MergeArgs mg, int nhb,
-                                                              int ncb, int ndb)
+                                                              int ncb)
 {
     if (a.gate && *a.gate == 0) return;
     constexpr int RKW = G * KW / 8;          // words per lane of the row passes' 8 lanes
@@ -883,11 +883,11 @@ void launch_mixed(const LevelArgs &a, cudaStream_t s)
     const int blocks = a.nviews * (2 * nhb + 2 * ncb + (a.npaths > 4 ? 4 * ndb : 0));
     constexpr int th = kStencilWarps * 32;
     if (a.Dw == a.Dws) {
-        if (a.v[0].lo) agg_mixed<G, KW, true, false><<<blocks, th, 0, s>>>(a, m, nhb, ncb, ndb);
-        else agg_mixed<G, KW, false, false><<<blocks, th, 0, s>>>(a, m, nhb, ncb, ndb);
+        if (a.v[0].lo) agg_mixed<G, KW, true, false><<<blocks, th, 0, s>>>(a, m, nhb, ncb);
+        else agg_mixed<G, KW, false, false><<<blocks, th, 0, s>>>(a, m, nhb, ncb);
     } else {
-        if (a.v[0].lo) agg_mixed<G, KW, true, true><<<blocks, th, 0, s>>>(a, m, nhb, ncb, ndb);
-        else agg_mixed<G, KW, false, true><<<blocks, th, 0, s>>>(a, m, nhb, ncb, ndb);
+        if (a.v[0].lo) agg_mixed<G, KW, true, true><<<blocks, th, 0, s>>>(a, m, nhb, ncb);
+        else agg_mixed<G, KW, false, true><<<blocks, th, 0, s>>>(a, m, nhb, ncb);
     }
 }
 
