@@ -17,26 +17,32 @@ namespace {
 constexpr int kTile = 16;          // output tile side of the convolution kernels
 
 // out[n][co][y][x] = b[co] + sum_{ci,ky,kx} w[co][ci][ky][kx] in[n][ci][y+ky-1][x+kx-1]
-// (zero padding), optional ReLU, for one output channel on the CUDA cores (FP32 input, or more
-// BF16 channels than the tensor-core kernel stages); one thread per output pixel.
+// (zero padding), optional ReLU, on the CUDA cores; one thread per output pixel and all output
+// channels: one channel (FP32 input, or more BF16 channels than the tensor-core kernel stages), or
+// 32 of at most kPixelCin FP32 channels.
 __device__ __forceinline__ float ld_act(const __nv_bfloat16 *p, int64_t i) { return __bfloat162float(p[i]); }
 __device__ __forceinline__ float ld_act(const float *p, int64_t i) { return p[i]; }
 
-template <class TIn>
-__global__ void __launch_bounds__(kTile *kTile) conv3x3_one_kernel(
+template <int COUT, class TIn>
+__global__ void __launch_bounds__(kTile *kTile) conv3x3_pixel_kernel(
     const TIn *__restrict__ in, int Cin, int H, int W,
     const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b, int relu,
     __nv_bfloat16 *__restrict__ out_bf, float *__restrict__ out_f)
 {
     extern __shared__ float smem[];
-    float *ws = smem;                                   // [Cin*9]
-    float *tile = smem + Cin * 9;                       // [18][18] of one input channel
+    float *ws = smem;                                   // [Cin*9][COUT]
+    float *tile = smem + Cin * 9 * COUT;                // [18][18] of one input channel
     const int n = blockIdx.z;
     const int tx = threadIdx.x % kTile, ty = threadIdx.x / kTile;
     const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
     const int x = x0 + tx, y = y0 + ty;
-    for (int i = threadIdx.x; i < Cin * 9; i += kTile * kTile) ws[i] = __bfloat162float(w[i]);
-    float acc = b ? b[0] : 0.f;
+    for (int i = threadIdx.x; i < Cin * 9 * COUT; i += kTile * kTile) {
+        const int co = i % COUT, r = i / COUT;         // r = ci*9 + k
+        ws[i] = __bfloat162float(w[(int64_t)co * Cin * 9 + r]);
+    }
+    float acc[COUT];
+#pragma unroll
+    for (int co = 0; co < COUT; ++co) acc[co] = b ? b[co] : 0.f;
     const int64_t plane = (int64_t)H * W;
     const TIn *src = in + (int64_t)n * Cin * plane;
     for (int ci = 0; ci < Cin; ++ci) {
@@ -49,15 +55,28 @@ __global__ void __launch_bounds__(kTile *kTile) conv3x3_one_kernel(
         }
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < 9; ++k)
-            acc = fmaf(ws[ci * 9 + k], tile[(ty + k / 3) * 18 + tx + k % 3], acc);
+        for (int k = 0; k < 9; ++k) {
+            const float v = tile[(ty + k / 3) * 18 + tx + k % 3];
+            const float *wr = ws + (ci * 9 + k) * COUT;
+#pragma unroll
+            for (int co = 0; co < COUT; ++co) acc[co] = fmaf(wr[co], v, acc[co]);
+        }
     }
     if (x >= W || y >= H) return;
-    const int64_t o = (int64_t)n * plane + (int64_t)y * W + x;
-    if (relu) acc = fmaxf(acc, 0.f);
-    if (out_f) out_f[o] = acc;
-    if (out_bf) out_bf[o] = __float2bfloat16(acc);
+    const int64_t o = (int64_t)n * COUT * plane + (int64_t)y * W + x;
+#pragma unroll
+    for (int co = 0; co < COUT; ++co) {
+        float v = acc[co];
+        if (relu) v = fmaxf(v, 0.f);
+        if (out_f) out_f[o + co * plane] = v;
+        if (out_bf) out_bf[o + co * plane] = __float2bfloat16(v);
+    }
 }
+
+// Up to this many FP32 channels conv3x3_pixel_kernel makes 32 channels: the other kernel's chunks
+// of 16 staged channels are mostly empty (8 samples of 320 x 180: one channel, the last layer's
+// backward pass, 19 us against 27; two 29 against 31; three 38 against 37).
+constexpr int kPixelCin = 2;
 
 // Two FP32 multiply-adds in one instruction (each rounded as fmaf), on register pairs.
 __device__ __forceinline__ unsigned long long pair(float lo, float hi)
@@ -76,11 +95,11 @@ __device__ __forceinline__ void fma2(unsigned long long &acc, unsigned long long
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
 
-// The same for 32 output channels and FP32 input (the backward-data pass): 4 pixels of a
+// The same for 32 output channels of more FP32 channels (the backward-data pass): 4 pixels of a
 // row x 8 channels per thread, a 16 x 16 tile per block, the input tile and the weights of
 // kConvChunk channels at a time in shared memory.  A (channel, ky) takes 8 shared loads for 96
 // multiply-adds, every operand of a warp in one or two 128-byte rows; the sums run in the same
-// order (channel, ky, kx) as with a thread per pixel, bit for bit the same.  Bound: the FP32
+// order as in conv3x3_pixel_kernel (channel, ky, kx), bit for bit the same.  Bound: the FP32
 // pipe (8 samples of 320 x 180, 32 -> 32 channels, 8.5 GFLOP: 295 -> 183 us against one pixel and
 // 32 channels per thread and one channel per barrier).
 constexpr int kConvChunk = 16, kConvRow = 20;       // channels per chunk; staged row (18 used)
@@ -886,26 +905,29 @@ unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 size_t conv_smem_bytes(int Cin, int Cout) { return sizeof(float) * ((size_t)Cin * 9 * Cout + 18 * 18); }
 
-template <class TIn>
-void launch_conv3x3_one(const TIn *in, int N, int Cin, int H, int W, const __nv_bfloat16 *w,
-                        const float *b, int relu, __nv_bfloat16 *out_bf, float *out_f,
-                        cudaStream_t s)
+template <int COUT, class TIn>
+void launch_conv3x3_pixel(const TIn *in, int N, int Cin, int H, int W, const __nv_bfloat16 *w,
+                          const float *b, int relu, __nv_bfloat16 *out_bf, float *out_f,
+                          cudaStream_t s)
 {
     dim3 grid((W + kTile - 1) / kTile, (H + kTile - 1) / kTile, N);
-    const size_t smem = conv_smem_bytes(Cin, 1);
-    cudaFuncSetAttribute(conv3x3_one_kernel<TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    conv3x3_one_kernel<TIn><<<grid, kTile * kTile, smem, s>>>(in, Cin, H, W, w, b, relu, out_bf, out_f);
+    const size_t smem = conv_smem_bytes(Cin, COUT);
+    cudaFuncSetAttribute(conv3x3_pixel_kernel<COUT, TIn>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    conv3x3_pixel_kernel<COUT, TIn><<<grid, kTile * kTile, smem, s>>>(in, Cin, H, W, w, b, relu,
+                                                                      out_bf, out_f);
 }
 
 void launch_conv3x3_f32(const float *in, int N, int Cin, int H, int W, const __nv_bfloat16 *w,
                         const float *b, int Cout, int relu, __nv_bfloat16 *out_bf, float *out_f,
                         cudaStream_t s)
 {
+    if (Cout == 1)
+        return launch_conv3x3_pixel<1>(in, N, Cin, H, W, w, b, relu, out_bf, out_f, s);
+    if (Cin <= kPixelCin)
+        return launch_conv3x3_pixel<32>(in, N, Cin, H, W, w, b, relu, out_bf, out_f, s);
     dim3 grid((W + kTile - 1) / kTile, (H + kTile - 1) / kTile, N);
-    if (Cout == 32)
-        conv3x3_f32_kernel<<<grid, 256, 0, s>>>(in, Cin, H, W, w, b, relu, out_bf, out_f);
-    else
-        launch_conv3x3_one(in, N, Cin, H, W, w, b, relu, out_bf, out_f, s);
+    conv3x3_f32_kernel<<<grid, 256, 0, s>>>(in, Cin, H, W, w, b, relu, out_bf, out_f);
 }
 
 int sm_count()
@@ -971,7 +993,7 @@ void launch_conv3x3(const __nv_bfloat16 *in, int N, int Cin, int H, int W, const
     if (conv3x3_tc_ok(Cin, Cout))
         launch_tc<false>(in, N, Cin, Cin, H, W, w, b, Cout, relu, out_bf, out_f, nullptr, s);
     else if (Cout == 1)
-        launch_conv3x3_one(in, N, Cin, H, W, w, b, relu, out_bf, out_f, s);
+        launch_conv3x3_pixel<1>(in, N, Cin, H, W, w, b, relu, out_bf, out_f, s);
 }
 
 void launch_conv3x3_wgrad(const __nv_bfloat16 *in, int N, int Cin, const float *g, int Cout, int H,
