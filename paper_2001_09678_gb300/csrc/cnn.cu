@@ -6,6 +6,7 @@
 // padding, 2 + D_top input channels (the top pyramid level's left and right images and
 // its full-range cost slice), 32 hidden channels with ReLU, 1 output channel: the
 // disparity at full resolution divided by D, at the top level's resolution.
+#include <algorithm>
 #include <cuda_bf16.h>
 
 #include "mpv_internal.cuh"
@@ -996,23 +997,40 @@ void launch_conv3x3(const __nv_bfloat16 *in, int N, int Cin, int H, int W, const
         launch_conv3x3_pixel<1>(in, N, Cin, H, W, w, b, relu, out_bf, out_f, s);
 }
 
+// Whether the tiled kernel takes a weight gradient.  Few input channels leave most of its threads
+// idle, and the general kernel is as fast or faster (us, general against tiled): 32 <- 1 channels
+// 13.0 / 13.1 with 60 tiles, 13.0 / 18.5 with 120, 64.7 / 69.2 with 1,920; 32 <- 2 channels
+// 16.0 / 13.3 with 60 tiles, 16.3 / 18.2 with 120, 28.8 / 33.6 with 320, 53.0 / 41.9 with 784;
+// 1 <- 1 channel 5.4 / 4.5 with 320, 11.5 / 12.9 with 1,920.  (Over 65,535 rows of tiles or
+// samples the general kernel's launch refuses the call.)
+bool wgrad_tiled(int Cin, int Cout, int64_t tiles, int64_t ty, int N)
+{
+    if ((Cout != 32 && Cout != 1) || Cin > kWgMaxCin || ty > 65535 || N > 65535 ||
+        tiles >= 0x7FFFFFFF)
+        return false;
+    const int64_t sms = sm_count();
+    if (Cout == 1) return Cin > 1 || tiles <= 3 * sms;
+    if (Cin == 1) return 5 * tiles <= 2 * sms;
+    return Cin > 2 || 5 * tiles <= 3 * sms || tiles > 3 * sms;
+}
+
 void launch_conv3x3_wgrad(const __nv_bfloat16 *in, int N, int Cin, const float *g, int Cout, int H,
                           int W, float *dw, float *db, cudaStream_t s)
 {
     const int64_t tx = (W + kTile - 1) / kTile, ty = (H + kTile - 1) / kTile, tiles = tx * ty * N;
-    if ((Cout == 32 || Cout == 1) && Cin <= kWgMaxCin && ty <= 65535 && N <= 65535 &&
-        tiles < 0x7FFFFFFF) {
+    if (wgrad_tiled(Cin, Cout, tiles, ty, N)) {
         const int64_t resident = (Cout == 1 ? 3 : 2) * (int64_t)sm_count();
         const unsigned blocks = (unsigned)(tiles < resident ? tiles : resident);
         size_t sm = sizeof(float) * ((size_t)kTile * kTile * (Cout == 1 ? 1 : kWgGS) +
                                      (size_t)Cin * kWgIS);
-        const int threads = (8 * Cin + 31) / 32 * 32;
+        // 256 threads at least, to stage the tiles (32 <- 3 channels or 1 <- 4 compute with one
+        // warp; with 32 threads 1 <- 4 channels took 34 instead of 14 us on 1,920 tiles)
+        const int threads = std::max(256, (8 * Cin + 31) / 32 * 32);
         if (Cout == 32) {
-            // (256 threads at least, to stage the tiles)
             cudaFuncSetAttribute(wgrad_tile_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sm);
-            wgrad_tile_kernel<4><<<blocks, threads < 256 ? 256 : threads, sm, s>>>(
-                in, Cin, g, H, W, (int)tx, (int)ty, (int)tiles, dw, db);
+            wgrad_tile_kernel<4><<<blocks, threads, sm, s>>>(in, Cin, g, H, W, (int)tx, (int)ty,
+                                                             (int)tiles, dw, db);
         } else {
             const size_t part = sizeof(float) * kWgSplit * 9 * (size_t)Cin;
             if (part > sm) sm = part;
