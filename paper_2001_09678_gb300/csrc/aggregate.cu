@@ -913,9 +913,13 @@ void launch_bytes(const LevelArgs &a, cudaStream_t s)
 
 }  // namespace
 
-// Jumps beyond two labels truncated, sums that fit a byte, no tiles.
+// Jumps beyond two labels truncated, sums that fit a byte, no tiles.  Not on narrow, tall levels
+// with windows of 16 labels: there the columns' chain is the launch, and a step of it is shorter
+// with 8 lanes of two labels and 16-bit sums (calls of two levels, windows of 7 labels, both
+// views: 64 x 1400 263 against 238 us, 128 x 800 164 against 160, 200 x 400 97 against 98).
 bool bytes_ok(const LevelArgs &a)
 {
+    if (a.Dws == 16 && a.v[0].lo && a.H >= 2 * a.W && a.W <= 256) return false;
     return a.radius <= 2 && a.Dws <= 64 && a.block_cut == 0 &&
            (int64_t)a.npaths * a.trunc <= 255 && packed_caps_ok(a, 1);
 }

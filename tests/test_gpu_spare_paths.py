@@ -27,7 +27,10 @@ CASES = [(5, 60, 5, 1, 0, 8, 1)] + \
         [(w, 44, 30, 2, 14, 8, 1) for w in range(41, 49, 2)] + \
         [(w, 41, 60, 2, 27, 8, 0) for w in range(74, 81, 2)] + \
         [(49, 45, 40, 1, 0, 8, 1), (94, 42, 90, 2, 45, 4, 1), (77, 44, 64, 1, 0, 8, 1),
-         (130, 43, 128, 2, 60, 8, 0)]
+         (130, 43, 128, 2, 60, 8, 0),
+         # narrow, tall levels with windows of 16 labels, and the first ones outside that rule
+         (20, 90, 14, 2, 7, 8, 1), (29, 58, 20, 2, 16, 4, 1), (29, 57, 20, 2, 16, 8, 0),
+         (256, 512, 14, 2, 7, 8, 1), (257, 514, 14, 2, 7, 8, 1)]
 
 
 @pytest.mark.parametrize("W,H,D,scales,window,paths,lr", CASES)
