@@ -118,18 +118,20 @@ def level_geometry():
 
 ALG_NOTE = {
     "cost": "images 2 B/px + cost write 1 B/node (cost stored as uint8: exact, costs <= 255)",
-    "aggregate": "cost read 1 B + summed-energy write 2 B per node (16-bit sums; byte sums "
-                 "write 1 B), window starts 2 B/px (the survey's B_alg reads a uint16 cost: "
-                 "2 B + 2 B, reported as frac_at_survey_bytes)",
-    "wta": "summed-energy read 2 B/node + window starts and map 2 B/px each",
+    "aggregate": "cost read 1 B + summed-energy write 1 B per node (byte sums; the layered merge "
+                 "2 B and more), window starts 2 B/px (the survey's B_alg reads a uint16 cost and "
+                 "writes a uint16 sum: 2 B + 2 B, reported as frac_at_survey_bytes)",
+    "wta": "2 B/node (a 16-bit sum, or the cost and a byte sum) + window starts and map 2 B/px "
+           "each",
 }
 
 
-def algorithmic_bytes(views=2, variant="plain", cost_bytes=1):
+def algorithmic_bytes(views=2, variant="plain", cost_bytes=1, sum_bytes=2):
     """Minimum HBM bytes per frame of each stage: the cost kernel reads both images and
     writes the cost volume (1 B/node: costs are <= 255); the aggregation reads it
-    (1 B/node) and writes the uint16 summed volume (2 B/node); winner-take-all reads
-    that (2 B/node) and writes the uint16 map.  The layered merge stores each pass
+    (1 B/node) and writes the summed volume (sum_bytes per node: 2, or 1 for the byte sums
+    of the energies' increments); winner-take-all reads 2 B/node (the 16-bit sums, or the
+    costs and the byte sums) and writes the uint16 map.  The layered merge stores each pass
     (2 B/node per direction) and reads the previous layer's pair (4 B/node per
     direction; the first layer reads the cost bytes), and its WTA reads the last pair."""
     merge, grad, lw = VARIANTS[variant]
@@ -151,7 +153,7 @@ def algorithmic_bytes(views=2, variant="plain", cost_bytes=1):
             agg += views * ((2 * n + 4 * n) + (layers - 1) * (8 * n + 4 * n) + img)
             wta += views * (4 * n + 2 * w * h + 2 * w * h)
         else:
-            agg += views * (cost_bytes * n + 2 * n + 2 * w * h + img)
+            agg += views * (cost_bytes * n + sum_bytes * n + 2 * w * h + img)
             wta += views * (2 * n + 2 * w * h + 2 * w * h)
     return dict(cost=cost, aggregate=agg, wta=wta), nodes
 
@@ -404,7 +406,8 @@ def run_mine(args):
     ok = np.array_equal(hd.numpy(), disp.cpu().numpy())
 
     # roofline of the dominant kernel (by device time over the timed region)
-    alg, nodes = algorithmic_bytes(variant=args.variant)
+    # (the default penalties' sums fit bytes: 8 paths, T = 30)
+    alg, nodes = algorithmic_bytes(variant=args.variant, sum_bytes=1)
     alg4, _ = algorithmic_bytes(variant=args.variant, cost_bytes=2)
     stage_ms = {k: v[0] for k, v in prof.items()}
     launches_per_frame = sum(v[1] for v in prof.values()) / prof_steps
@@ -453,7 +456,8 @@ def run_mine(args):
                 "alg_bytes_per_node": ALG_NOTE[dom],
                 "frac_at_survey_bytes": round(achieved4 / peak, 4),
                 # the whole path: every stage's algorithmic bytes of one frame over the
-                # frame time (the survey's whole-path figure reads a uint16 cost: the second)
+                # frame time (the survey's whole-path figure reads a uint16 cost and moves
+                # uint16 sums: the second)
                 "whole_path": {"alg_bytes_per_step": int(sum(alg.values())),
                                "frac": round(sum(alg.values()) / (ms_per_step * 1e-3) / 1e9 / peak, 4),
                                "frac_at_survey_bytes": round(sum(alg4.values()) / (ms_per_step * 1e-3)

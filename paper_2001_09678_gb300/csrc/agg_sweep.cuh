@@ -14,9 +14,9 @@
 // window starts and intensities a chunk ahead in registers, from which each lane prepares the
 // slope and shift of two steps.
 //
-// Bound: issue on large levels (141 instructions per step of 8 paths), the chain of a row step on
-// others.  Both views, 8 paths, against 8 lanes, prefix scans by shuffles and 16-bit sums:
-// 1280x720, 32 labels, windows 712 -> 421 us; 640x360 178 -> 130 us; 320x180 without windows
+// Bound: issue and L1 on large levels (138 instructions per step of 8 paths; 64 and 73 %), the
+// chain of a row step on others.  Both views, 8 paths, against 8 lanes, prefix scans by shuffles
+// and 16-bit sums: 1280x720, 32 labels, windows 712 -> 421 us; 640x360 178 -> 130 us; 320x180 without windows
 // 83 -> 49 us.  8 lanes for the rows (109 instructions per step of 4 paths) 636 instead of 612 us
 // per frame; windows that moved by 2 labels through shuffles 631 us; 12 to 28 resident warps per
 // SM within 5 %.

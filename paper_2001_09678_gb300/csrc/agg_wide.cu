@@ -20,10 +20,10 @@
 //
 // Measured on a GB300, 1280x720, 128 labels, 8 paths, both views: 785 us (8 lanes 826 us)
 // against 4,600 us for one warp per path on int32 scans with 32-bit reductions into 16-bit
-// sums (agg_general, kept for what lies outside the rule in wide_shape).  Bound: DRAM and the
-// reductions (4.4 GB of DRAM traffic, 5.4 TB/s; the volumes are four times the L2, and eight
-// directions read C and add to E), issue slots 75 % active.  4 and 8 cost stages measure the
-// same; the step unrolled by 4 lost to instruction fetches.
+// sums (agg_general, kept for what lies outside the rule in wide_shape).  Bound: HBM (4.1 GB
+// of DRAM traffic, 5.2 TB/s; the volumes are four times the L2, and eight directions read C and
+// add to E); issue slots 61 %, ALU pipe 45 % active.  4 and 8 cost stages measure the same; the
+// step unrolled by 4 lost to instruction fetches.
 #include "volume_layout.cuh"
 
 namespace mpv {

@@ -904,8 +904,8 @@ void launch_bytes(const LevelArgs &a, cudaStream_t s)
     case 16: launch_mixed<4, 2>(a, s); return;
     case 32: launch_mixed<4, 4>(a, s); return;
     // (48 labels, 1920x1080 with windows: 2,088 -> 1,050 us, of which half the sums' bytes and
-    // whole-sector accesses (bytes48_of) are most; 123 instructions per step of 8 paths, L1
-    // 84 % busy)
+    // whole-sector accesses (bytes48_of) are most; 122 instructions per step of 8 paths, L1
+    // 82 % busy)
     case 48: launch_bytes_kw<4, 6>(a, s); return;
     default: launch_bytes_kw<8, 4>(a, s); return;
     }

@@ -327,7 +327,7 @@ __device__ __forceinline__ void cost_body(const LevelArgs &a, int uspan_max, int
 
     const int stride = ORD == 1 ? 4 * a.wide_g * a.wide_nq : Dws;
     if (ORD == 1) {   // this segment's byte sums start at zero, the bytes of no label at cost 255
-        const int64_t at = ((int64_t)y * W + x0) * stride;     // a multiple of 32
+        const int64_t at = ((int64_t)y * W + x0) * stride;     // a multiple of 16
         const int n16 = npx * (stride / 16);
         uint4 *ez = (uint4 *)(V.E + at), *cz = (uint4 *)(V.C + at);
         const uint32_t f = 0xFFFFFFFFu;

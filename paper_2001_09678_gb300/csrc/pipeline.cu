@@ -325,7 +325,7 @@ LevelArgs level_args(const mpv_params &p, const PairPlan &pp, uint8_t *base, int
     }
     if (sums == kSumsBytes && l == 0 && wide_shape(a, a.wide_g, a.wide_nq)) {
         // C and E share the region of C and S (adjacent, 3 Dws bytes per pixel, no fewer than
-        // two wide volumes); E starts on 8 bytes
+        // two wide volumes); E starts on 16 bytes
         const size_t vol = (size_t)a.W * a.H * (4 * a.wide_g * a.wide_nq);
         for (int v = 0; v < pp.nviews; ++v) a.v[v].E = a.v[v].C + vol;
     } else {
